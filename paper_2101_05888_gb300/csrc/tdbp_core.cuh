@@ -70,7 +70,8 @@ constexpr int BAR_CONS = 1;             // named barrier of the consumer warps
 
 enum { MODE_FORWARD = 0, MODE_OFFSET_GRAD = 1 };
 // group descriptor flags: the group ends its stage / is the last one
-enum { GD_STAGE_END = 1, GD_LAST = 2 };
+// or holds a pair whose legs take the exact per-pixel form (see leg_series)
+enum { GD_STAGE_END = 1, GD_LAST = 2, GD_EXACT = 4 };
 
 // record fields of one (ping, channel) pair, in the order of the float4 a
 // consumer loads: {2R_R, |R_R|^2}, {|R_R|, 2 frac u_ref - 1/2, phase [rad], scale},
@@ -86,7 +87,8 @@ enum {
 };
 // pair flags: the whole tile lies inside the transmitter / receiver beam;
 // the transmitter / receiver leg refracts into the sediment for some pixel
-enum { FL_TX_FULL = 1, FL_RX_FULL = 2, FL_T_REFR = 4, FL_R_REFR = 8 };
+// the column series does not hold for one of the legs (see leg_series)
+enum { FL_TX_FULL = 1, FL_RX_FULL = 2, FL_T_REFR = 4, FL_R_REFR = 8, FL_EXACT = 16 };
 // With the seabed refraction model the record has two more blocks of RF_N
 // fields after the first sixteen (the receiver leg's, then the
 // transmitter leg's), in place of the beam and motion fields:
@@ -133,6 +135,11 @@ struct KParams {
     double z_int, refr_n;
     float refr_nf, refr_r2, refr_M, refr_isM, refr_tol;
     float hx, hy, hz;       // half extents of a tile's pixel-centre box [m]
+    // column series (see leg_series): offsets +-(k + 1/2) step of the slots from
+    // the column's centre and their squares, packed over k = (0, 1), (2, 3);
+    // radians per half sample; |R| from which the series holds
+    float2 ypos[PX / 4], yneg[PX / 4], ysq[PX / 4];
+    float ph_hs, series_rmin;
     int U, npos, npos_pad, seglen, seg_align, slot_bytes;
     int accumulate, atomic_out, skip_copies;
     unsigned long long wait_ns;
@@ -699,6 +706,65 @@ __device__ __forceinline__ float fixed_dot(float tx, float ty, float dx, float d
     return DIM3 ? fmaf(tx, dx, __fmul_rn(ty, dy)) : __fmul_rn(tx, dx);
 }
 
+// Column series.  A thread's PX pixels lie on a line (slots along y in 2D, z
+// in 3D), so a leg's length along it, r(y) = sqrt(r0^2 + 2 b y + y^2) with y
+// from the line's centre (r0 = |R + d0| there, b = (R + d0) . axis), is a
+// smooth function of one variable: r(y) = r0 + c1 y + c2 y^2 + ..., where
+// squaring gives c1 = b / r0, c2 = (1 - c1^2) / (2 r0), c3 = -c1 c2 / r0,
+// c4 = -(2 c1 c3 + c2^2) / (2 r0).  One rsqrt and one rcp then serve PX pixels
+// (they had bound the pixel loop: with four SFU operations an update the SFU
+// pipe was 66 % busy, the busiest of the SM's pipes).  The first term left out is
+// r0 |C5| (y / r0)^5 with |C5| <= 0.1 (the Gegenbauer polynomial
+// (P3 - P5) / 9); the host bounds it by 5e-6 rad of carrier phase, a third
+// of what rounding the path to FP32 costs, which holds from series_rmin
+// (6 .. 10 m in 2D, 2 m over a 3D column) on; pairs nearer than that take the
+// exact form at every pixel.
+// c[0] = r0 - |R| (the differential path at the line's centre), c[1 .. 4] as
+// above.  a0 = 2R.d0 + |d0|^2, b = (R + d0) . axis, n2 = |R|^2, n = |R|.  The
+// root and the quotient of c[0] take a Newton step each: the SFU's 1e-7
+// relative would cost 1e-5 rad and more over a tile's path span, and here the
+// steps are shared by PX pixels.
+__device__ __forceinline__ void leg_series(float a0, float b, float n2, float n, float* c) {
+    const float sm = n2 + a0;
+    const float rs = rsqrt_sfu(sm), hr = 0.5f * rs;
+    float r0 = sm * rs;
+    r0 = fmaf(hr, fmaf(-r0, r0, sm), r0);
+    const float den = r0 + n, rc = rcp_sfu(den), q0 = a0 * rc;
+    c[0] = fmaf(rc, fmaf(-den, q0, a0), q0);
+    c[1] = b * rs;
+    c[2] = hr * fmaf(-c[1], c[1], 1.f);
+    const float q = c[1] * rs;
+    c[3] = -(q * c[2]);
+    c[4] = fmaf(-q, c[3], -(hr * c[2] * c[2]));
+}
+// The series at the slots at +-(2h + 1/2, 2h + 3/2) steps from the centre:
+// fwd: slots PX/2 + 2h, + 1; back: PX/2 - 1 - 2h, - 1 (even and odd parts shared).
+__device__ __forceinline__ void series_quad(const KParams& p, const float* c, int h, float2& fwd, float2& back) {
+    const float2 ev = ffma2(ffma2(make_float2(c[4], c[4]), p.ysq[h], make_float2(c[2], c[2])), p.ysq[h],
+                            make_float2(c[0], c[0]));
+    const float2 od = ffma2(make_float2(c[3], c[3]), p.ysq[h], make_float2(c[1], c[1]));
+    fwd = ffma2(od, p.ypos[h], ev);
+    back = ffma2(od, p.yneg[h], ev);
+}
+// 2R.d0 + |d0|^2 and (R + d0) . axis at the line's centre from a record's 2R;
+// (dx, dy): the column's fixed offsets (dy in 3D only), dvc its centre's, d2c = |d0|^2
+template <bool DIM3>
+__device__ __forceinline__ float centre_a(float tx, float ty, float tz, float dx, float dy, float dvc, float d2c) {
+    return DIM3 ? fmaf(tz, dvc, fmaf(ty, dy, fmaf(tx, dx, d2c))) : fmaf(ty, dvc, fmaf(tx, dx, d2c));
+}
+template <bool DIM3>
+__device__ __forceinline__ float centre_b(float ty, float tz, float dvc) {
+    return fmaf(0.5f, DIM3 ? tz : ty, dvc);
+}
+// differential path of one leg at one pixel (the exact form): dvs the slot's
+// offset, d2 = |d|^2, X = fixed_dot
+template <bool DIM3>
+__device__ __forceinline__ float leg_exact(float ty, float tz, float n2, float n, float X, float dvs, float d2) {
+    const float a = __fadd_rn(fmaf(DIM3 ? tz : ty, dvs, d2), X);
+    const float sm = n2 + a;
+    return a * rcp_sfu(fmaf(sm, rsqrt_sfu(sm), n));
+}
+
 // Shared-memory size and launch geometry, host side.
 struct Layout {
     int U, npos, seglen, align, slot_bytes;
@@ -743,6 +809,8 @@ template <typename ET, bool DIM3, int MODE, bool BEAM, bool MOTION, bool REFRACT
 __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant__ CUtensorMap tmap, const KParams p) {
     using T = Tile<DIM3>;
     static_assert(!REFRACT || (!BEAM && !MOTION), "refraction: without the beam or receiver motion");
+    // the forward pass over straight legs takes the column series
+    constexpr bool SERIES = MODE == MODE_FORWARD && !REFRACT && !MOTION;
     constexpr int KREC = REFRACT ? NREC_REFR : NREC;   // record fields
     // FP16 Farrow rows for 16-bit echoes in the forward pass; otherwise rows
     // of FP32 E0, E1 and BF16 E2, E3
@@ -922,6 +990,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
                     rc[F_OFF] = __int_as_float(base - seg_start);
                     rc[F_SCALE] = p.scale ? p.scale[qv] : 1.0f;
                     rc[F_PING] = __int_as_float(iv);
+                    if (SERIES && !(fminf(rc[F_NT], rc[F_NR]) >= p.series_rmin)) flv |= FL_EXACT;
                     rc[F_FLAGS] = __int_as_float(REFRACT ? rfl : flv);
                     if constexpr (!REFRACT) {
 #pragma unroll
@@ -969,6 +1038,10 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
         auto emit = [&](int rs, int pr0, int ng, int flags, int ss) {
             const int b = G % NBUF;
             if (G >= NBUF && !mbar_wait_bounded(smem_u32(&eempty[b]), ((G / NBUF) - 1) & 1, p.wait_ns)) fail();
+            if (SERIES) {
+                const bool exact = lane < ng && (__float_as_int(rec[(rs * PAIRS + pr0 + lane) * KREC + F_FLAGS]) & FL_EXACT);
+                if (__any_sync(0xffffffffu, exact)) flags |= GD_EXACT;
+            }
             if (!failed && ng > 0) {
                 const float* rc = rec + rs * PAIRS * KREC;
                 unsigned char* eb = ebuf + (size_t)b * GROUP * ebuf_pair;
@@ -1075,7 +1148,14 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
     // differential range of the current ping, held as pairs of slots (2k, 2k+1)
     // for the packed geometry.  The offsets are formed exactly as the adjoint
     // kernel forms them, so both evaluate identical paths.
-    float2 dvp[PX / 2], d2p[PX / 2], dTp[PX / 2];
+    // (column series: the centre's offset dvc and |d0|^2, and the transmitter's
+    // series in half samples)
+    float2 dvp[SERIES ? 1 : PX / 2], d2p[SERIES ? 1 : PX / 2], dTp[SERIES ? 1 : PX / 2];
+    float dvc = 0.f, d2c0 = 0.f, sT[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    // column series: the image accumulators in two parts, sum s cos and sum s sin,
+    // each a packed FMA an update (the rotation's cross terms are resolved once,
+    // when the tile is written)
+    float2 accs[SERIES ? PX : 1];
 #define PXS(arr, s) (((s) & 1) ? arr[(s) >> 1].y : arr[(s) >> 1].x)
     float2 acc[PX];                       // forward: image accumulators; gradient: G(x)
     float rsum[MODE == MODE_OFFSET_GRAD ? PX : 1];
@@ -1088,13 +1168,19 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
         dv0 = DIM3 ? opaque((float)((tz0 + lz - cz) * p.dz)) : dyv_c;
         dvstep = DIM3 ? opaque((float)p.dz) : opaque((float)(4.0 * p.dy));
         const float d2c = fixed_d2<DIM3>(dxv, dyv_c);
+        dvc = fmaf(0.5f * (PX - 1), dvstep, dv0);
+        d2c0 = fmaf(dvc, dvc, d2c);
 #pragma unroll
         for (int s = 0; s < PX; ++s) {
             T::pixel(ct, s, lx, ly, lz);
-            const float dvs = fmaf((float)s, dvstep, dv0);
-            PXS(dvp, s) = dvs;
-            PXS(d2p, s) = fmaf(dvs, dvs, d2c);
-            PXS(dTp, s) = 0.f;
+            if constexpr (!SERIES) {
+                const float dvs = fmaf((float)s, dvstep, dv0);
+                PXS(dvp, s) = dvs;
+                PXS(d2p, s) = fmaf(dvs, dvs, d2c);
+                PXS(dTp, s) = 0.f;
+            } else {
+                accs[s] = make_float2(0.f, 0.f);
+            }
             if (MODE == MODE_FORWARD) {
                 acc[s] = make_float2(0.f, 0.f);
             } else {
@@ -1380,6 +1466,96 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
         }
     };
 
+    // Column-series forms of the above (forward pass, straight legs).  One
+    // update: the row of half-sample coordinate t = v + 1.5 2^23, g = v - rint(v),
+    // the carrier phase x; sum s cos(x) and sum s sin(x).
+    auto update = [&](auto masked, const int s, const float tj, const float g, const float x, const bool seen,
+                      const unsigned char* erow) {
+        constexpr bool MASKED = decltype(masked)::value;
+        const unsigned char* erow_b = erow + npos_pad * NH * 16;
+        const unsigned pos = row_index((unsigned)(__float_as_int(tj) - (__float_as_int(FLOOR_MAGIC) - NH * p.U)),
+                                       (unsigned)(NH * p.npos - 1), p.status);
+        float sn, cs;
+        sincos_sfu(x, sn, cs);
+        if (MASKED && !seen) {
+            sn = 0.f;
+            cs = 0.f;
+        }
+        const float2 gg2 = make_float2(g, g);
+        const float4 e01 = *reinterpret_cast<const float4*>(erow + pos * 16);
+        float2 v;
+        if constexpr (E16) {
+            const float2 e2 = *reinterpret_cast<const float2*>(erow_b + pos * 8);
+            v = ffma2(e2, gg2, make_float2(e01.z, e01.w));
+        } else {
+            const float4 e23 = *reinterpret_cast<const float4*>(erow_b + pos * 16);
+            v = ffma2(make_float2(e23.z, e23.w), gg2, make_float2(e23.x, e23.y));
+            v = ffma2(v, gg2, make_float2(e01.z, e01.w));
+        }
+        v = ffma2(v, gg2, make_float2(e01.x, e01.y));
+        acc[s] = ffma2(v, make_float2(cs, cs), acc[s]);
+        accs[SERIES ? s : 0] = ffma2(v, make_float2(sn, sn), accs[SERIES ? s : 0]);
+    };
+    // the beam test of slot s (MASKED pairs)
+    auto slot_seen = [&](const int s, const float4 q0, const float* rot, uint32_t rmask_needed) {
+        const float dvs = fmaf((float)s, dvstep, dv0);
+        const float wx = fmaf(0.5f, q0.x, dxv);
+        const float wy = DIM3 ? fmaf(0.5f, q0.y, dyv_c) : fmaf(0.5f, q0.y, dvs);
+        const float wz = DIM3 ? fmaf(0.5f, q0.z, dvs) : 0.5f * q0.z;
+        return ((tmask >> s) & 1u) && (!rmask_needed || beam_sees(p, wx, wy, wz, rot));
+    };
+    auto centre_series = [&](const float4 q, const float n, float* c) {
+        leg_series(centre_a<DIM3>(q.x, q.y, q.z, dxv, dyv_c, dvc, d2c0), centre_b<DIM3>(q.y, q.z, dvc), q.w, n, c);
+    };
+    auto pixels_series = [&](auto masked, auto direct, const float4 q0, const float4 q1, const float* rot,
+                             uint32_t rmask_needed, const unsigned char* erow) {
+        constexpr bool MASKED = decltype(masked)::value;
+        constexpr bool DIRECT = decltype(direct)::value;
+        float c[5];
+        centre_series(q0, q1.x, c);
+        // 2 (u - floor u_ref) - 1/2 along the line, both legs, in half samples
+        c[0] = fmaf(c[0], p.hs_c, sT[0] + q1.y);
+#pragma unroll
+        for (int k = 1; k < 5; ++k) c[k] = fmaf(c[k], p.hs_c, sT[k]);
+        const float phk = fmaf(-q1.y, p.ph_hs, q1.z);      // carrier phase [rad] = v ph_hs + phk
+        const float2 magic2 = make_float2(FLOOR_MAGIC, FLOOR_MAGIC);
+        auto pair = [&](const float2 v, const int s0, const int s1) {
+            float2 x2 = ffma2(v, make_float2(p.ph_hs, p.ph_hs), make_float2(phk, phk));
+            const float2 t = fadd2(v, magic2);
+            const float2 g2 = fsub2(v, fsub2(t, magic2));
+            if constexpr (!DIRECT) x2 = reduce_phase2(x2);
+            update(masked, s0, t.x, g2.x, x2.x, !MASKED || slot_seen(s0, q0, rot, rmask_needed), erow);
+            update(masked, s1, t.y, g2.y, x2.y, !MASKED || slot_seen(s1, q0, rot, rmask_needed), erow);
+        };
+#pragma unroll
+        for (int h = 0; h < PX / 4; ++h) {
+            float2 fwd, back;
+            series_quad(p, c, h, fwd, back);
+            pair(fwd, PX / 2 + 2 * h, PX / 2 + 2 * h + 1);
+            pair(back, PX / 2 - 1 - 2 * h, PX / 2 - 2 - 2 * h);
+        }
+    };
+    // pairs too near for the series: both legs at every pixel
+    auto pixels_exact = [&](auto direct, const float4 q0, const float4 q1, const float4 q2, const float nT,
+                            const float* rot, uint32_t rmask_needed, const unsigned char* erow) {
+        constexpr bool DIRECT = decltype(direct)::value;
+        const float phk = fmaf(-q1.y, p.ph_hs, q1.z);
+        const float XR = fixed_dot<DIM3>(q0.x, q0.y, dxv, dyv_c), XT = fixed_dot<DIM3>(q2.x, q2.y, dxv, dyv_c);
+        const float d2c = fixed_d2<DIM3>(dxv, dyv_c);
+#pragma unroll
+        for (int s = 0; s < PX; ++s) {
+            const float dvs = fmaf((float)s, dvstep, dv0), d2 = fmaf(dvs, dvs, d2c);
+            const float D = leg_exact<DIM3>(q0.y, q0.z, q0.w, q1.x, XR, dvs, d2) +
+                            leg_exact<DIM3>(q2.y, q2.z, q2.w, nT, XT, dvs, d2);
+            const float v = fmaf(D, p.hs_c, q1.y);
+            float x = fmaf(v, p.ph_hs, phk);
+            if constexpr (!DIRECT) x = reduce_phase(x);
+            const float t = __fadd_rn(v, FLOOR_MAGIC);
+            update(std::integral_constant<bool, BEAM>{}, s, t, v - __fadd_rn(t, -FLOOR_MAGIC), x,
+                   !BEAM || slot_seen(s, q0, rot, rmask_needed), erow);
+        }
+    };
+
     // ---- the groups in the order the producer emits them
     bool aborted = false;
     int prev_ping = -1;
@@ -1454,25 +1630,32 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
                     ftr1 = tr1;
                     ftr2 = tr2;
                 }
+                if constexpr (SERIES) {
+                    centre_series(q2, tNT, sT);
+#pragma unroll
+                    for (int k = 0; k < 5; ++k) sT[k] *= p.hs_c;
+                }
 #pragma unroll
                 for (int s = 0; s < PX; ++s) {
-                    const float a = __fadd_rn(fmaf(tTv, PXS(dvp, s), PXS(d2p, s)), X);
-                    const float sm = tNT2 + a;
-                    const float den = fmaf(sm, rsqrt_sfu(sm), tNT);
-                    PXS(dTp, s) = a * rcp_sfu(den);
-                    if (REFRACT && trefr) {
-                        if ((bmask >> s) & 1u) {
-                            if (!DIM3) refr_rho(tr0, a, rhoT, drhoT);
-                            float b, db;
-                            slot_depth(s, b, db);
-                            float uxi, ua;
-                            PXS(dTp, s) = refr_leg_diff(p, tr0, tr1, tr2, rhoT, drhoT, b, db, r_br, uxi, ua);
-                        } else {
-                            PXS(dTp, s) += tr2.w;
+                    if constexpr (!SERIES) {
+                        const float a = __fadd_rn(fmaf(tTv, PXS(dvp, s), PXS(d2p, s)), X);
+                        const float sm = tNT2 + a;
+                        const float den = fmaf(sm, rsqrt_sfu(sm), tNT);
+                        PXS(dTp, s) = a * rcp_sfu(den);
+                        if (REFRACT && trefr) {
+                            if ((bmask >> s) & 1u) {
+                                if (!DIM3) refr_rho(tr0, a, rhoT, drhoT);
+                                float b, db;
+                                slot_depth(s, b, db);
+                                float uxi, ua;
+                                PXS(dTp, s) = refr_leg_diff(p, tr0, tr1, tr2, rhoT, drhoT, b, db, r_br, uxi, ua);
+                            } else {
+                                PXS(dTp, s) += tr2.w;
+                            }
                         }
                     }
                     if (BEAM && !(flags & FL_TX_FULL)) {
-                        const float dvs = PXS(dvp, s);
+                        const float dvs = fmaf((float)s, dvstep, dv0);
                         const float wx = fmaf(0.5f, tT0, dxv);
                         const float wy = DIM3 ? fmaf(0.5f, tT1, dyv_c) : fmaf(0.5f, tT1, dvs);
                         const float wz = DIM3 ? fmaf(0.5f, tT2, dvs) : 0.5f * tT2;
@@ -1487,7 +1670,28 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
             using F_ = std::integral_constant<bool, false>;
             using T_ = std::integral_constant<bool, true>;
             using B_ = std::integral_constant<bool, BEAM>;
-            if (!BEAM || (flags & (FL_TX_FULL | FL_RX_FULL)) == (FL_TX_FULL | FL_RX_FULL)) {
+            if constexpr (SERIES) {
+                const bool full = !BEAM || (flags & (FL_TX_FULL | FL_RX_FULL)) == (FL_TX_FULL | FL_RX_FULL);
+                const uint32_t rmn = (flags & FL_RX_FULL) ? 0u : 1u;
+                if (gflags & GD_EXACT) {
+                    const float4 q2 = hr[2];
+                    const float nT = hr[3].x;
+                    if (p.phase_direct)
+                        pixels_exact(T_{}, q0, q1, q2, nT, rot, rmn, erow);
+                    else
+                        pixels_exact(F_{}, q0, q1, q2, nT, rot, rmn, erow);
+                } else if (full) {
+                    if (p.phase_direct)
+                        pixels_series(F_{}, T_{}, q0, q1, rot, 0u, erow);
+                    else
+                        pixels_series(F_{}, F_{}, q0, q1, rot, 0u, erow);
+                } else {
+                    if (p.phase_direct)
+                        pixels_series(B_{}, T_{}, q0, q1, rot, rmn, erow);
+                    else
+                        pixels_series(B_{}, F_{}, q0, q1, rot, rmn, erow);
+                }
+            } else if (!BEAM || (flags & (FL_TX_FULL | FL_RX_FULL)) == (FL_TX_FULL | FL_RX_FULL)) {
                 if (p.phase_direct)
                     pixels(F_{}, T_{}, q0, q1, rot, 0u, erow, q6, q7, hr, rfl);
                 else
@@ -1515,6 +1719,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
         T::pixel(ct, s, lx, ly, lz);
         const int ix = tx0 + lx, iy = ty0 + ly, iz = tz0 + lz;
         if (ix >= p.nx || iy >= p.ny || iz >= p.nz) continue;
+        if constexpr (SERIES) acc[s] = make_float2(acc[s].x - accs[s].y, acc[s].y + accs[s].x);
         float2* dst = p.image + ((size_t)iz * p.ny + iy) * p.nx + ix;
         if (p.atomic_out) {
             atomicAdd(dst, acc[s]);

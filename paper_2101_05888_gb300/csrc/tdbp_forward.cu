@@ -19,7 +19,18 @@ int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long min_ctas, S
     const double dmax = std::sqrt(hx * hx + hy * hy + hz * hz);
     // with seabed refraction a leg's length in water metres is Lipschitz with
     // constant max(1, n), n = c / c_s (a straight segment costs at most that much)
-    const bool refract = h->c_sed > 0.0;
+    if (h->c_sed > 0.0 && (h->beam_tan > 0.0 || h->has_vel)) {
+        set_error("the refraction model does not combine with receiver motion or a beam");
+        return SAS_ERR_UNSUPPORTED;
+    }
+    // no pixel layer below the interface, or no step in the sound speed: every
+    // leg is straight, and the straight kernels (about four times as fast, with
+    // the column series) give the same image (layers as layer_z forms them)
+    bool refract = h->c_sed > 0.0 && h->c_sed != h->sig.c;
+    if (refract) {
+        volatile double z_off = (double)(nz - 1) * dz;   // rounded by itself, as layer_z does
+        refract = std::max(g.z0, g.z0 + z_off) > h->z_int;
+    }
     const double n_refr = refract ? h->sig.c / h->c_sed : 1.0;
     const int U = (int)std::ceil(2.0 * std::max(1.0, n_refr) * dmax * h->sig.fs / h->sig.c) + 2;
     const int elem = (h->echo_dtype == SAS_ECHO_C32_F16 || h->echo_dtype == SAS_ECHO_C32_BF16) ? 4 : 8;
@@ -99,6 +110,21 @@ int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long min_ctas, S
     prm.hx = (float)hx;
     prm.hy = (float)hy;
     prm.hz = (float)hz;
+    // column series (leg_series): the slots' offsets and the range from which
+    // the term left out, r |C5| (y / r)^5 with |C5| <= 0.1 at the line's ends,
+    // stays below 5e-6 rad of carrier phase (and the line short against r)
+    const double ystep = std::fabs(dim3 ? dz : 4.0 * g.dy), ymax = 0.5 * (PX - 1) * ystep;
+    const double sgn = (dim3 ? dz : g.dy) < 0.0 ? -1.0 : 1.0;
+    for (int k = 0; k < PX / 2; ++k) {
+        const float y = (float)(sgn * (k + 0.5) * ystep);
+        float2 &a = prm.ypos[k / 2], &b = prm.yneg[k / 2], &c = prm.ysq[k / 2];
+        (k & 1 ? a.y : a.x) = y;
+        (k & 1 ? b.y : b.x) = -y;
+        (k & 1 ? c.y : c.x) = y * y;
+    }
+    prm.ph_hs = (float)(M_PI * h->sig.fc / h->sig.fs);
+    const double err_m = 5e-6 * h->sig.c / (2.0 * M_PI * std::max(std::fabs(h->sig.fc), h->sig.fs));
+    prm.series_rmin = (float)(dmax + std::max(8.0 * ymax, std::pow(0.1 * std::pow(ymax, 5.0) / err_m, 0.25)));
     prm.skip_copies = h->debug_skip_copies;
     prm.wait_ns = (unsigned long long)(h->debug_wait_ms > 0 ? h->debug_wait_ms : 4000) * 1000000ull;
     const long long ntiles = (long long)prm.tiles_x * prm.tiles_y * prm.tiles_z;
