@@ -13,6 +13,9 @@
 // atomics.
 #include "tdbp_core.cuh"
 
+#include <algorithm>
+#include <cmath>
+
 namespace sas {
 
 int launch_offset_grad(sas_geometry_t h, const sas_grid& g, const float2* grad_image, double* grad_offsets,
@@ -139,7 +142,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) adjoint_kernel(const KParams p, c
                             leg_series(centre_a<DIM3>(tT0, tT1, tT2, dxv, dyv_c, dvc, fmaf(dvc, dvc, d2c)),
                                        centre_b<DIM3>(tT1, tT2, dvc), nT2, nT, sT);
 #pragma unroll
-                            for (int q = 0; q < 5; ++q) sT[q] *= p.hs_c;
+                            for (int q = 0; q < 5; ++q) sT[q] *= p.hs_s;
                         }
                         // seabed refraction of the transmitter leg
                         const bool trefr = REFRACT && (rfl_s[pr] & FL_T_REFR);
@@ -183,9 +186,9 @@ __global__ void __launch_bounds__(NTHREADS, 2) adjoint_kernel(const KParams p, c
                         float c[5];
                         leg_series(centre_a<DIM3>(tRx, tRy, tRz, dxv, dyv_c, dvc, fmaf(dvc, dvc, d2c)),
                                    centre_b<DIM3>(tRy, tRz, dvc), nR2, nR, c);
-                        c[0] = fmaf(c[0], p.hs_c, sT[0] + ufc);
+                        c[0] = fmaf(c[0], p.hs_s, sT[0] + ufc);
 #pragma unroll
-                        for (int q = 1; q < 5; ++q) c[q] = fmaf(c[q], p.hs_c, sT[q]);
+                        for (int q = 1; q < 5; ++q) c[q] = fmaf(c[q], p.hs_s, sT[q]);
 #pragma unroll
                         for (int h = 0; h < PX / 4; ++h) {
                             float2 back;
@@ -258,7 +261,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) adjoint_kernel(const KParams p, c
                                 const float eps = fmaf(dvar[s], vv, Km) * rs;         // u_R . v / c
                                 D = D * fmaf(eps, eps - 1.f, 1.f);                   // / (1 + eps)
                             }
-                            v = fmaf(D, p.hs_c, ufc);
+                            v = fmaf(D, series ? p.hs_s : p.hs_c, ufc);
                         }
                         // carrier phase [rad]
                         float ph = series ? fmaf(v, p.ph_hs, fmaf(-ufc, p.ph_hs, phr)) : fmaf(D, p.wfc_c, phr);
@@ -319,7 +322,360 @@ __global__ void __launch_bounds__(NTHREADS, 2) adjoint_kernel(const KParams p, c
     }
 }
 
+// ----------------------------------------------------------------------------
+// 2D, straight legs, stop-and-hop, no beam: one warp per (ping, channel) pair.
+//
+// The kernel above adds eight FP32 values an update with shared-memory atomics,
+// which have no native form here (a compare-and-swap loop each: 14 G updates/s)
+// and separates scatter, FIR and clearing by block barriers.  Here a warp owns
+// its pair's accumulator rows, so that a row is updated by a plain load, add
+// and store; the lanes of one instruction only have to hit different rows.
+// They lie along one axis of the tile, two pixels apart, on the axis along which
+// the two-way path changes faster: where neighbouring lanes' half-sample
+// coordinates differ by at least one (bounded per pair from the unit vectors
+// at the tile's centre and the tile's radius over the ranges) their rows are distinct.
+// Pairs without that guarantee, or too near for the column series, take the
+// slow form: both legs at every pixel, lanes with equal rows one after the other.
+// Each lane walks lines of 32 pixels along the other axis with the column
+// series of the forward pass, and keeps the sums of its current row in registers
+// until the row changes.
+// 128 pings x 8 RX -> 512 x 480: 17.5 ms before, 0.83 ms now (304 G updates/s);
+// issue 66 % and the shared-memory pipe 60 % busy (adding every pixel to its
+// row at once: 1.07 ms, that pipe 83 %).
+constexpr int AT = 64;                    // tile edge [pixels]
+constexpr int AIS = AT + 1;               // image row stride: lanes two rows or two columns apart, two-way conflicts
+constexpr int AW = 8;                     // warps a block, one pair each
+constexpr int APB = 4;                    // pairs whose records a warp forms at once
+// record fields kept, and after them the low parts of 2R (x, y), |R|^2, |R| of both legs
+enum { AF_RXL = F_OFF + 1, AF_RYL, AF_NR2L, AF_NRL, AF_TXL, AF_TYL, AF_NT2L, AF_NTL, AREC };
+static_assert(AREC % 4 == 0, "records are read by 16-byte loads");
+constexpr int ALINE = 32;                 // pixels of a line (a lane's series)
+enum { AF_Y = 1, AF_SLOW = 2 };           // lanes lie along y; slow form
+
+// One leg along a line of pixels (leg_series with its centre term in two parts).
+// The lines are four times as long as a forward thread's and lie up to 45 pixels
+// from the tile's centre, and an error of a pair's reference terms moves a whole
+// tile coherently: with 2R, |R| and the quotient rounded to FP32 the inner
+// products of the transpose were off by 2e-5 (1e-5 in the smaller tiles of the
+// forward pass), so those terms carry their low parts.  (tA, tB), (tAl, tBl): 2R
+// along the lanes' and the line's axis; oA, oB: the line's centre, also in two
+// parts (a pixel spacing rounded to FP32 moves the tile's edge by 1e-8 m, 1e-5
+// rad); (n2, n2l), (n, nl): |R|^2 and |R|.
+struct LineLeg {
+    float Dh, Dl, c1, c2, c3, c4;
+};
+__device__ __forceinline__ float two_sum(float a, float b, float& err) {
+    const float s = __fadd_rn(a, b), bb = __fsub_rn(s, a);
+    err = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    return s;
+}
+__device__ __forceinline__ LineLeg line_leg(float tA, float tB, float tAl, float tBl, dfl oAd, dfl oBd, float n2,
+                                            float n, float n2l, float nl) {
+    const float oA = oAd.hi, oB = oBd.hi;
+    const float p1 = __fmul_rn(tA, oA), p2 = __fmul_rn(tB, oB), d2 = fmaf(oA, oA, oB * oB);
+    float e1, e2, e3, e4;
+    const float a = two_sum(two_sum(p1, p2, e1), d2, e2);            // 2R.d + |d|^2
+    const float al = fmaf(tA, oA, -p1) + fmaf(tB, oB, -p2) + (e1 + e2) + fmaf(tAl, oA, tBl * oB) +
+                     fmaf(tA, oAd.lo, tB * oBd.lo);
+    const float sm = two_sum(n2, a, e3), sml = e3 + (n2l + al);       // |R + d|^2
+    float rs = rsqrt_sfu(sm);
+    rs = fmaf(0.5f * rs, fmaf(-(sm * rs), rs, 1.f), rs);
+    const float hr = 0.5f * rs, r0 = sm * rs;
+    const float r0l = hr * (fmaf(-r0, r0, sm) + sml);                 // |R + d| = r0 + r0l
+    const float den = two_sum(r0, n, e4), rc = rcp_sfu(den);
+    LineLeg L;
+    L.Dh = a * rc;
+    L.Dl = rc * (fmaf(-den, L.Dh, a) + fmaf(-(e4 + (r0l + nl)), L.Dh, al));
+    L.c1 = fmaf(0.5f, tB, oB) * rs;
+    L.c2 = hr * fmaf(-L.c1, L.c1, 1.f);
+    const float q = L.c1 * rs;
+    L.c3 = -(q * L.c2);
+    L.c4 = fmaf(-q, L.c3, -(hr * L.c2 * L.c2));
+    return L;
+}
+
+inline size_t adjoint2d_smem(int npos) {
+    return sizeof(float2) * AT * AIS + sizeof(float4) * NH * TAPS +
+           (size_t)AW * (sizeof(float4) * 2 * NH * npos + sizeof(float) * APB * AREC);
+}
+
+// p: with this kernel's tiles, window (U, npos) and series_rmin (lines of ALINE)
+__global__ void __launch_bounds__(32 * AW, 2) adjoint2d_kernel(const KParams p, const float2* __restrict__ img,
+                                                              float2* __restrict__ eadj, int Ns) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    const int nrow = NH * p.npos;
+    float4* coef_s = reinterpret_cast<float4*>(smem);                        // [NH][TAPS] x NP
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    float4* rows = coef_s + NH * TAPS + (size_t)warp * 2 * nrow;             // two planes: powers 0, 1 and 2, 3
+    float4* recs = coef_s + NH * TAPS + (size_t)AW * 2 * nrow;
+    float* rec = reinterpret_cast<float*>(recs) + warp * APB * AREC;
+    float2* im = reinterpret_cast<float2*>(reinterpret_cast<float*>(recs) + AW * APB * AREC);   // [AT][AIS]
+
+    const int ntiles = p.tiles_x * p.tiles_y;
+    const int tile = blockIdx.x % ntiles, split = blockIdx.x / ntiles;
+    const int tx0 = (tile % p.tiles_x) * AT, ty0 = (tile / p.tiles_x) * AT;
+    const int nx = min(AT, p.nx - tx0), ny = min(AT, p.ny - ty0);
+    const long long q0 = (long long)min(p.P, split * p.pings_per_split) * p.C;
+    const long long q1 = (long long)min(p.P, (split + 1) * p.pings_per_split) * p.C;
+    for (int i = threadIdx.x; i < AT * AIS; i += 32 * AW) {
+        const int y = i / AIS, x = i - y * AIS;
+        im[i] = x < nx && y < ny ? img[(size_t)(ty0 + y) * p.nx + tx0 + x] : make_float2(0.f, 0.f);
+    }
+    for (int i = lane; i < 2 * nrow; i += 32) rows[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (threadIdx.x < NH * TAPS)
+        coef_s[threadIdx.x] = *reinterpret_cast<const float4*>(&p.coef->c[threadIdx.x / TAPS][threadIdx.x % TAPS][0]);
+    __syncthreads();
+    const double X0 = p.x0 + (tx0 + 0.5 * (AT - 1)) * p.dx, Y0 = p.y0 + (ty0 + 0.5 * (AT - 1)) * p.dy;
+    const float2 dx2 = df_split(p.dx), dy2 = df_split(p.dy);             // pixel spacings as double-floats
+    const float2 hx2 = df_split(p.dx * (double)p.hs_s), hy2 = df_split(p.dy * (double)p.hs_s);   // in half samples
+    const dfl ddx = dfl{opaque(dx2.x), opaque(dx2.y)}, ddy = dfl{opaque(dy2.x), opaque(dy2.y)};
+    const dfl hdx = dfl{opaque(hx2.x), opaque(hx2.y)}, hdy = dfl{opaque(hy2.x), opaque(hy2.y)};
+    const float fdx = ddx.hi, fdy = ddy.hi;
+    // k pixels, k a half-integer below 64: the product in two parts
+    auto times = [](float k, dfl d) {
+        const float q = __fmul_rn(k, d.hi);
+        return dfl{q, fmaf(k, d.hi, -q) + k * d.lo};
+    };
+    const float2 a_ = df_split(X0), b_ = df_split(Y0), c_ = df_split(p.z0);
+    const dfl X0d[3] = {dfl{a_.x, a_.y}, dfl{b_.x, b_.y}, dfl{c_.x, c_.y}};
+    const float2 magic2 = make_float2(FLOOR_MAGIC, FLOOR_MAGIC);
+
+    // adds a[0 .. 3] to a row (lanes' rows distinct)
+    auto add_row = [&](const unsigned pos, const float2* a) {
+        const float4 e = rows[pos], f = rows[nrow + pos];
+        const float2 s0 = fadd2(make_float2(e.x, e.y), a[0]), s1 = fadd2(make_float2(e.z, e.w), a[1]);
+        const float2 s2 = fadd2(make_float2(f.x, f.y), a[2]), s3 = fadd2(make_float2(f.z, f.w), a[3]);
+        rows[pos] = make_float4(s0.x, s0.y, s1.x, s1.y);
+        rows[nrow + pos] = make_float4(s2.x, s2.y, s3.x, s3.y);
+    };
+    auto powers = [&](const float2 w, const float g, float2* a) {   // g^p w
+        const float2 gg = make_float2(g, g);
+        a[0] = w;
+        a[1] = fmul2(w, gg);
+        a[2] = fmul2(a[1], gg);
+        a[3] = fmul2(a[2], gg);
+    };
+    // the row and weighted value of one pixel: half-sample coordinate v (t = v +
+    // 1.5 2^23, g = v - rint v), phase x, image value I
+    auto row_of = [&](const float t) {
+        return row_index((unsigned)(__float_as_int(t) - (__float_as_int(FLOOR_MAGIC) - NH * p.U)), (unsigned)(nrow - 1),
+                         p.status);
+    };
+    auto weighted = [&](const float x, const float2 I) {   // I exp(-j x)
+        float sn, cs;
+        sincos_sfu(x, sn, cs);
+        return make_float2(fmaf(I.x, cs, I.y * sn), fmaf(I.y, cs, -I.x * sn));
+    };
+
+    // the warp's pairs: q0 + warp, + AW, ...
+    for (long long qb = q0 + warp; qb < q1; qb += AW * APB) {
+        const int cnt = (int)min((long long)APB, (q1 - qb + AW - 1) / AW);
+        if (lane < cnt) {
+            const int q = (int)(qb + AW * lane), i = q / p.C;
+            float* rc = rec + lane * AREC;
+            const PairGeoDF G = pair_geo_df(p, X0d, q, i);
+            rc[F_OFF] = __int_as_float(pair_record_df(p, G, rc, 1));
+#pragma unroll
+            for (int leg = 0; leg < 2; ++leg) {
+                // the record's fields are the double-floats' rounded values
+                const dfl* g = leg ? G.T : G.R;
+                const dfl n2 = df_add(df_add(df_mul(g[0], g[0]), df_mul(g[1], g[1])), df_mul(g[2], g[2]));
+                const dfl n1 = df_sqrt(n2);
+                float* lo = rc + (leg ? AF_TXL : AF_RXL);
+                const float* hi = rc + (leg ? F_TX : F_RX);
+                const float nh = rc[leg ? F_NT : F_NR];
+                lo[0] = fmaf(2.f, g[0].lo, fmaf(2.f, g[0].hi, -hi[0]));
+                lo[1] = fmaf(2.f, g[1].lo, fmaf(2.f, g[1].hi, -hi[1]));
+                lo[2] = (n2.hi - hi[3]) + n2.lo;
+                lo[3] = (n1.hi - nh) + n1.lo;
+            }
+            // change of the half-sample coordinate between neighbouring lanes
+            // (two pixels), at least, along either axis
+            const float nT = rc[F_NT], nR = rc[F_NR], dmax = sqrtf(p.hx * p.hx + p.hy * p.hy);
+            const float turn = dmax / fmaxf(nT - dmax, 1e-6f) + dmax / fmaxf(nR - dmax, 1e-6f);
+            const float sx = fabsf(0.5f * rc[F_TX] / nT + 0.5f * rc[F_RX] / nR);
+            const float sy = fabsf(0.5f * rc[F_TY] / nT + 0.5f * rc[F_RY] / nR);
+            const float vx = 2.f * fabsf(fdx) * p.hs_s * (sx - turn), vy = 2.f * fabsf(fdy) * p.hs_s * (sy - turn);
+            int fl = vy >= vx ? AF_Y : 0;
+            // (the margin covers FP32 rounding of the coordinates; a range that is
+            // not finite compares false)
+            if (!(fmaxf(vx, vy) >= 1.01f && fminf(nT, nR) >= p.series_rmin)) fl |= AF_SLOW;
+            rc[F_FLAGS] = __int_as_float(fl);
+        }
+        __syncwarp();
+        for (int j = 0; j < cnt; ++j) {
+            const float4* rc = reinterpret_cast<const float4*>(rec + j * AREC);
+            const float4 r0 = rc[0], r1 = rc[1], r2 = rc[2], r3 = rc[3], r4 = rc[4], r5 = rc[5];
+            const int fl = __float_as_int(r3.z);
+            const bool ay = fl & AF_Y;
+            const float dA = ay ? fdy : fdx, dB = ay ? fdx : fdy;
+            const float rA = ay ? r0.y : r0.x, rB = ay ? r0.x : r0.y, tA = ay ? r2.y : r2.x, tB = ay ? r2.x : r2.y;
+            const int nA = ay ? ny : nx, nB = ay ? nx : ny, strA = ay ? AIS : 1, strB = ay ? 1 : AIS;
+            const float phk = fmaf(-r1.y, p.ph_hs, r1.z);
+            if (!(fl & AF_SLOW)) {
+#pragma unroll 1
+                for (int l4 = 0; l4 < 4; ++l4) {
+                    const int a0i = l4 & 1, b0 = (l4 >> 1) * ALINE;
+                    if (a0i >= nA || b0 >= nB) continue;
+                    const dfl oA = times(2 * lane + a0i - 0.5f * (AT - 1), ay ? ddy : ddx);
+                    const dfl oB = times(b0 + 0.5f * (ALINE - 1) - 0.5f * (AT - 1), ay ? ddx : ddy);
+                    const LineLeg T = line_leg(tA, tB, ay ? r5.y : r5.x, ay ? r5.x : r5.y, oA, oB, r2.w, r3.x, r5.z, r5.w);
+                    const LineLeg R = line_leg(rA, rB, ay ? r4.y : r4.x, ay ? r4.x : r4.y, oA, oB, r0.w, r1.x, r4.z, r4.w);
+                    float pl;
+                    const float ph = two_sum(T.Dh, R.Dh, pl);
+                    pl = pl + (T.Dl + R.Dl);
+                    // half-sample coordinate v0 and carrier phase x0 at the line's centre, the phase
+                    // from whole cycles removed
+                    const float v0 = fmaf(ph, p.hs_s, r1.y);
+                    const float cy = __fmul_rn(ph, p.k_fc_c.x);
+                    const float fr = __fsub_rn(cy, __fsub_rn(__fadd_rn(cy, FLOOR_MAGIC), FLOOR_MAGIC));
+                    const float x0 = fmaf(fr + fmaf(ph, p.k_fc_c.x, -cy) + fmaf(ph, p.k_fc_c.y, pl * p.k_fc_c.x),
+                                          TWO_PI_F, r1.z);
+                    // the series in pixels from the line's centre (exact half-integers)
+                    const dfl hB = ay ? hdx : hdy;
+                    const float c1s = T.c1 + R.c1, hB2 = hB.hi * dB, hB3 = hB2 * dB;
+                    const float c1 = fmaf(c1s, hB.hi, c1s * hB.lo), c2 = (T.c2 + R.c2) * hB2;
+                    const float c3 = (T.c3 + R.c3) * hB3, c4 = (T.c4 + R.c4) * (hB3 * dB);
+                    const float2* ip = im + (2 * lane + a0i) * strA + b0 * strB;
+                    const int nb = min(ALINE, nB - b0);
+                    // the lane's current row and its sums: pixels along the line often share a row
+                    // (the path changes slower along it), and a row is added when it is left
+                    unsigned cur = 0u;
+                    float2 sum[4];
+                    auto put = [&](const unsigned pos, const float2 w, const float g, const bool first) {
+                        float2 a[4];
+                        powers(w, g, a);
+                        if (first || pos != cur) {
+                            if (!first) add_row(cur, sum);
+                            cur = pos;
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) sum[q] = a[q];
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) sum[q] = fadd2(sum[q], a[q]);
+                        }
+                        __syncwarp();
+                    };
+                    float2 y = make_float2(-0.5f * (ALINE - 1), 1.f - 0.5f * (ALINE - 1));
+#pragma unroll 2
+                    for (int k = 0; k < nb; k += 2) {
+                        // along the line from its centre: dv half samples, phase x0 + dv ph_hs
+                        float2 dv = ffma2(make_float2(c4, c4), y, make_float2(c3, c3));
+                        dv = ffma2(dv, y, make_float2(c2, c2));
+                        dv = fmul2(ffma2(dv, y, make_float2(c1, c1)), y);
+                        y = fadd2(y, make_float2(2.f, 2.f));
+                        // (reduced: unreduced phases cost the SFU 1.5e-7 of their size, 1e-5 here)
+                        const float2 x = reduce_phase2(ffma2(dv, make_float2(p.ph_hs, p.ph_hs), make_float2(x0, x0)));
+                        const float2 v = fadd2(dv, make_float2(v0, v0));
+                        const float2 t = fadd2(v, magic2), g = fsub2(v, fsub2(t, magic2));
+                        const float2 I0 = ip[0], I1 = ip[strB];      // (zero past the tile's last pixel)
+                        ip += 2 * strB;
+                        const float2 w0 = weighted(x.x, I0), w1 = weighted(x.y, I1);
+                        put(row_of(t.x), w0, g.x, k == 0);
+                        put(row_of(t.y), w1, g.y, false);
+                    }
+                    add_row(cur, sum);
+                    __syncwarp();
+                }
+            } else {
+                for (int a = lane; a - lane < nA; a += 32) {
+                    const float oA = (a - 0.5f * (AT - 1)) * dA;
+                    for (int b = 0; b < nB; ++b) {
+                        const float oB = (b - 0.5f * (AT - 1)) * dB, d2 = fmaf(oA, oA, oB * oB);
+                        const float dR = leg_exact<false>(rB, 0.f, r0.w, r1.x, rA * oA, oB, d2);
+                        const float dT = leg_exact<false>(tB, 0.f, r2.w, r3.x, tA * oA, oB, d2);
+                        const float v = fmaf(dR + dT, p.hs_s, r1.y);
+                        const float x = reduce_phase(fmaf(v, p.ph_hs, phk));
+                        const float t = __fadd_rn(v, FLOOR_MAGIC), g = v - __fadd_rn(t, -FLOOR_MAGIC);
+                        const unsigned pos = row_of(t);
+                        const float2 w = weighted(x, im[a * strA + b * strB]);
+                        // lanes with the same row in turn
+                        const int turn = __popc(__match_any_sync(0xffffffffu, pos) & ((1u << lane) - 1u));
+                        const int turns = __reduce_max_sync(0xffffffffu, turn);
+                        float2 s[4];
+                        powers(w, g, s);
+                        for (int k = 0; k <= turns; ++k) {
+                            if (turn == k) add_row(pos, s);
+                            __syncwarp();
+                        }
+                    }
+                }
+            }
+            // transposed FIR: out[t] = sum_m sum_h sum_p coef[h][m][p] A_p[2 (t - m) + h], three
+            // consecutive samples a lane (each row is read once and used for three)
+            const long long base = __float_as_int(r3.w), row = qb + AW * j;
+            for (int t0 = 3 * lane; t0 < p.npos + TAPS - 1; t0 += 96) {
+                float2 o[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+#pragma unroll
+                for (int h = 0; h < NH; ++h) {
+                    float4 e[3], f[3];   // rows of positions t0 - m + (0, 1, 2)
+                    auto load = [&](int n, float4& a, float4& b) {
+                        const bool in = n >= 0 && n < p.npos;
+                        a = in ? rows[NH * n + h] : make_float4(0.f, 0.f, 0.f, 0.f);
+                        b = in ? rows[nrow + NH * n + h] : make_float4(0.f, 0.f, 0.f, 0.f);
+                    };
+                    load(t0 + 1, e[1], f[1]);
+                    load(t0 + 2, e[2], f[2]);
+#pragma unroll
+                    for (int m = 0; m < TAPS; ++m) {
+                        load(t0 - m, e[0], f[0]);
+                        const float4 c = coef_s[h * TAPS + m];
+#pragma unroll
+                        for (int k = 0; k < 3; ++k) {
+                            o[k] = ffma2(make_float2(c.x, c.x), make_float2(e[k].x, e[k].y), o[k]);
+                            o[k] = ffma2(make_float2(c.y, c.y), make_float2(e[k].z, e[k].w), o[k]);
+                            o[k] = ffma2(make_float2(c.z, c.z), make_float2(f[k].x, f[k].y), o[k]);
+                            o[k] = ffma2(make_float2(c.w, c.w), make_float2(f[k].z, f[k].w), o[k]);
+                        }
+                        e[2] = e[1]; f[2] = f[1];
+                        e[1] = e[0]; f[1] = f[0];
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 3; ++k) {
+                    const long long idx = base + t0 + k;
+                    if (t0 + k < p.npos + TAPS - 1 && idx >= 0 && idx < Ns && (o[k].x != 0.f || o[k].y != 0.f))
+                        atomicAdd(eadj + row * Ns + idx, o[k]);
+                }
+            }
+            __syncwarp();
+            for (int i = lane; i < 2 * nrow; i += 32) rows[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            __syncwarp();
+        }
+        __syncwarp();   // the records are rewritten
+    }
+}
+
 }  // namespace core
+
+// the rule for adjoint2d_kernel: straight stop-and-hop legs in 2D without a beam
+// (its tiles differ from the forward pass's, so beam decisions would not agree bit
+// for bit).  The accumulator rows of its eight warps take 150 KB at the
+// coarsest pixel spacing prepare() takes.  Sets the launch's parameters in S.
+static bool adjoint2d_plan(sas_geometry_t h, const sas_grid& g, core::Setup& S, size_t& smem) {
+    using namespace core;
+    KParams& p = S.prm;
+    if (g.nz > 1 || p.refract || p.beam || p.vel) return false;
+    const double hx = 0.5 * (AT - 1) * std::fabs(g.dx), hy = 0.5 * (AT - 1) * std::fabs(g.dy);
+    const double dmax = std::sqrt(hx * hx + hy * hy);
+    const int U = (int)std::ceil(2.0 * dmax * h->sig.fs / h->sig.c) + 2;
+    smem = adjoint2d_smem(2 * U + 1);
+    if (smem > 200 * 1024) return false;
+    p.U = U;
+    p.npos = 2 * U + 1;
+    p.hx = (float)hx;
+    p.hy = (float)hy;
+    const double ymax = 0.5 * (ALINE - 1) * std::max(std::fabs(g.dx), std::fabs(g.dy));
+    p.series_rmin = (float)series_range(h, dmax, ymax);
+    p.tiles_x = (g.nx + AT - 1) / AT;
+    p.tiles_y = (g.ny + AT - 1) / AT;
+    // (loading a tile and clearing the rows costs about four pairs' time)
+    const long long ntiles = (long long)p.tiles_x * p.tiles_y;
+    p.pings_per_split = pick_pings_per_split(ntiles, h->P, h->C, 2LL * sm_count(), 4.0, 4864);
+    p.nsplit = (h->P + p.pings_per_split - 1) / p.pings_per_split;
+    S.blocks = (int)(ntiles * p.nsplit);
+    return true;
+}
 
 static int launch_linear_adjoint(sas_geometry_t h, const sas_grid& g, const float2* img, float2* eadj,
                                  cudaStream_t st) {
@@ -332,6 +688,13 @@ static int launch_linear_adjoint(sas_geometry_t h, const sas_grid& g, const floa
         return SAS_ERR_UNSUPPORTED;
     }
     SAS_CUDA(cudaMemsetAsync(eadj, 0, sizeof(float2) * (size_t)h->P * h->C * h->Ns, st));
+    size_t smem2d = 0;
+    if (adjoint2d_plan(h, g, S, smem2d)) {
+        SAS_CUDA(cudaFuncSetAttribute(core::adjoint2d_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem2d));
+        core::adjoint2d_kernel<<<S.blocks, 32 * core::AW, smem2d, st>>>(S.prm, img, eadj, h->Ns);
+        SAS_CUDA(cudaGetLastError());
+        return SAS_OK;
+    }
     const int krec = S.prm.refract ? (int)core::NREC_REFR : (int)core::NREC;
     const size_t smem = sizeof(float2) * core::GROUP * NH * S.prm.npos * NP + sizeof(float) * krec * core::PAIRS +
                         sizeof(float) * NH * TAPS * NP + 2 * sizeof(int) * core::PAIRS;

@@ -137,9 +137,10 @@ struct KParams {
     float hx, hy, hz;       // half extents of a tile's pixel-centre box [m]
     // column series (see leg_series): offsets +-(k + 1/2) step of the slots from
     // the column's centre and their squares, packed over k = (0, 1), (2, 3);
-    // radians per half sample; |R| from which the series holds
+    // half samples per metre and radians per half sample, rounded as a pair;
+    // |R| from which the series holds
     float2 ypos[PX / 4], yneg[PX / 4], ysq[PX / 4];
-    float ph_hs, series_rmin;
+    float hs_s, ph_hs, series_rmin;
     int U, npos, npos_pad, seglen, seg_align, slot_bytes;
     int accumulate, atomic_out, skip_copies;
     unsigned long long wait_ns;
@@ -719,6 +720,10 @@ __device__ __forceinline__ float fixed_dot(float tx, float ty, float dx, float d
 // of what rounding the path to FP32 costs, which holds from series_rmin
 // (6 .. 10 m in 2D, 2 m over a 3D column) on; pairs nearer than that take the
 // exact form at every pixel.
+// Measured against an rsqrt and a rcp a pixel: 250 pings x 24 RX -> 1500 x 1101,
+// BF16: 13.53 -> 12.31 ms; 196 x 64 -> 256 x 224 x 56, FP16: 47.3 -> 43.5 ms;
+// 512 x 32 -> 4096^2, complex64: 338.6 -> 332.4 ms (there the shared-memory pipe
+// binds now, 79 % busy with 32 bytes of Farrow rows an update).
 // c[0] = r0 - |R| (the differential path at the line's centre), c[1 .. 4] as
 // above.  a0 = 2R.d0 + |d0|^2, b = (R + d0) . axis, n2 = |R|^2, n = |R|.  The
 // root and the quotient of c[0] take a Newton step each: the SFU's 1e-7
@@ -1514,9 +1519,9 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
         float c[5];
         centre_series(q0, q1.x, c);
         // 2 (u - floor u_ref) - 1/2 along the line, both legs, in half samples
-        c[0] = fmaf(c[0], p.hs_c, sT[0] + q1.y);
+        c[0] = fmaf(c[0], p.hs_s, sT[0] + q1.y);
 #pragma unroll
-        for (int k = 1; k < 5; ++k) c[k] = fmaf(c[k], p.hs_c, sT[k]);
+        for (int k = 1; k < 5; ++k) c[k] = fmaf(c[k], p.hs_s, sT[k]);
         const float phk = fmaf(-q1.y, p.ph_hs, q1.z);      // carrier phase [rad] = v ph_hs + phk
         const float2 magic2 = make_float2(FLOOR_MAGIC, FLOOR_MAGIC);
         auto pair = [&](const float2 v, const int s0, const int s1) {
@@ -1547,7 +1552,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
             const float dvs = fmaf((float)s, dvstep, dv0), d2 = fmaf(dvs, dvs, d2c);
             const float D = leg_exact<DIM3>(q0.y, q0.z, q0.w, q1.x, XR, dvs, d2) +
                             leg_exact<DIM3>(q2.y, q2.z, q2.w, nT, XT, dvs, d2);
-            const float v = fmaf(D, p.hs_c, q1.y);
+            const float v = fmaf(D, p.hs_s, q1.y);
             float x = fmaf(v, p.ph_hs, phk);
             if constexpr (!DIRECT) x = reduce_phase(x);
             const float t = __fadd_rn(v, FLOOR_MAGIC);
@@ -1633,7 +1638,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
                 if constexpr (SERIES) {
                     centre_series(q2, tNT, sT);
 #pragma unroll
-                    for (int k = 0; k < 5; ++k) sT[k] *= p.hs_c;
+                    for (int k = 0; k < 5; ++k) sT[k] *= p.hs_s;
                 }
 #pragma unroll
                 for (int s = 0; s < PX; ++s) {
@@ -1755,6 +1760,18 @@ inline void tile_dims(int dim3, int& TXs, int& TYs, int& TZs) {
 // Fills the launch description for grid g; min_ctas: aim for at least this
 // many CTAs by splitting the pings of each tile (0 = never split); mode: the
 // tdbp_kernel mode the launch runs (sets the Farrow row format).
+// range from which the column series holds on lines of half length ymax, for a
+// point within dmax of the tile centre: the term left out, r |C5| (y / r)^5 with
+// |C5| <= 0.1, stays below 5e-6 rad of carrier phase there (and the line
+// is short against r)
+double series_range(sas_geometry_t h, double dmax, double ymax);
+
+// Pings per block when `ntiles` tiles of P pings x C channels run on `slots`
+// resident blocks: the split with the least time in whole waves of blocks, where a
+// block costs its pairs plus `overhead` pairs; at most max_blocks blocks (or
+// one a tile).
+int pick_pings_per_split(long long ntiles, int P, int C, long long slots, double overhead, long long max_blocks);
+
 int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long min_ctas, Setup& S, bool need_echo = true,
             int mode = MODE_FORWARD);
 

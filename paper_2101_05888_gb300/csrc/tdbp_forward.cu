@@ -8,6 +8,26 @@
 namespace sas {
 namespace core {
 
+double series_range(sas_geometry_t h, double dmax, double ymax) {
+    const double err_m = 5e-6 * h->sig.c / (2.0 * M_PI * std::max(std::fabs(h->sig.fc), h->sig.fs));
+    return dmax + std::max(8.0 * ymax, std::pow(0.1 * std::pow(ymax, 5.0) / err_m, 0.25));
+}
+
+int pick_pings_per_split(long long ntiles, int P, int C, long long slots, double overhead, long long max_blocks) {
+    int best = P;
+    double best_cost = 0.0;
+    for (long long s = 1; s <= P && (s == 1 || s * ntiles <= max_blocks); ++s) {
+        const int pps = (int)((P + s - 1) / s);
+        const long long blocks = ntiles * ((P + pps - 1) / pps);
+        const double cost = (double)((blocks + slots - 1) / slots) * ((double)pps * C + overhead);
+        if (s == 1 || cost < best_cost) {
+            best_cost = cost;
+            best = pps;
+        }
+    }
+    return best;
+}
+
 int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long min_ctas, Setup& S, bool need_echo, int mode) {
     int TXs, TYs, TZs;
     tile_dims(dim3, TXs, TYs, TZs);
@@ -110,9 +130,7 @@ int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long min_ctas, S
     prm.hx = (float)hx;
     prm.hy = (float)hy;
     prm.hz = (float)hz;
-    // column series (leg_series): the slots' offsets and the range from which
-    // the term left out, r |C5| (y / r)^5 with |C5| <= 0.1 at the line's ends,
-    // stays below 5e-6 rad of carrier phase (and the line short against r)
+    // column series (leg_series): the slots' offsets and its least range
     const double ystep = std::fabs(dim3 ? dz : 4.0 * g.dy), ymax = 0.5 * (PX - 1) * ystep;
     const double sgn = (dim3 ? dz : g.dy) < 0.0 ? -1.0 : 1.0;
     for (int k = 0; k < PX / 2; ++k) {
@@ -122,9 +140,27 @@ int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long min_ctas, S
         (k & 1 ? b.y : b.x) = -y;
         (k & 1 ? c.y : c.x) = y * y;
     }
-    prm.ph_hs = (float)(M_PI * h->sig.fc / h->sig.fs);
-    const double err_m = 5e-6 * h->sig.c / (2.0 * M_PI * std::max(std::fabs(h->sig.fc), h->sig.fs));
-    prm.series_rmin = (float)(dmax + std::max(8.0 * ymax, std::pow(0.1 * std::pow(ymax, 5.0) / err_m, 0.25)));
+    // The series' paths become half samples, and those radians: rounding the two
+    // factors each by itself would scale the phase (up to 500 rad over a tile) by
+    // up to 7e-8, so of the FP32 values next to 2 fs/c (two ulps: 1e-5 half
+    // samples over a tile) the one is taken whose product with the rounded
+    // radians per half sample comes nearest to 2 pi fc/c.
+    {
+        const double hs = 2.0 * h->sig.fs / h->sig.c, w = 2.0 * M_PI * h->sig.fc / h->sig.c;
+        float f = (float)hs;
+        for (int k = 0; k < 2; ++k) f = std::nextafter(f, 0.0f);
+        double best = -1.0;
+        for (int k = 0; k < 5; ++k, f = std::nextafter(f, INFINITY)) {
+            const float r = (float)(w / (double)f);
+            const double err = std::fabs((double)f * (double)r - w);
+            if (best < 0.0 || err < best) {
+                best = err;
+                prm.hs_s = f;
+                prm.ph_hs = r;
+            }
+        }
+    }
+    prm.series_rmin = (float)series_range(h, dmax, ymax);
     prm.skip_copies = h->debug_skip_copies;
     prm.wait_ns = (unsigned long long)(h->debug_wait_ms > 0 ? h->debug_wait_ms : 4000) * 1000000ull;
     const long long ntiles = (long long)prm.tiles_x * prm.tiles_y * prm.tiles_z;
