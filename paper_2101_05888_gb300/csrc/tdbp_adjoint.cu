@@ -67,11 +67,9 @@ __global__ void __launch_bounds__(NTHREADS, 2) adjoint_kernel(const KParams p, c
     for (int t = tid; t < alen; t += NTHREADS) A[t] = make_float2(0.f, 0.f);
     if (tid < NH * TAPS * NP) coef_s[tid] = (&p.coef->c[0][0][0])[tid];
 
-    // without refraction and motion: the forward pass's column series (leg_series)
-    const bool series = !REFRACT && !p.vel;
     const bool consumer = warp > 0;
     const int ct = tid - 32;
-    float dxv = 0.f, dyv_c = 0.f, d2c = 0.f, r_d2h = 0.f, dvc = 0.f, sT[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
+    float dxv = 0.f, dyv_c = 0.f, d2c = 0.f, r_d2h = 0.f;
     float dvar[PX], dT[PX];
     float2 G[PX];
     if (consumer) {
@@ -85,7 +83,6 @@ __global__ void __launch_bounds__(NTHREADS, 2) adjoint_kernel(const KParams p, c
         const float dvstep = DIM3 ? (float)p.dz : (float)(4.0 * p.dy);
         d2c = fixed_d2<DIM3>(dxv, dyv_c);
         r_d2h = REFRACT ? fixed_d2<true>(dxv, dyv_c) : 0.f;
-        dvc = fmaf(0.5f * (PX - 1), dvstep, dv0);
 #pragma unroll
         for (int s = 0; s < PX; ++s) {
             T::pixel(ct, s, lx, ly, lz);
@@ -138,12 +135,6 @@ __global__ void __launch_bounds__(NTHREADS, 2) adjoint_kernel(const KParams p, c
                         const float nT2 = __shfl_sync(0xffffffffu, r[F_NT2], pr);
                         const float nT = __shfl_sync(0xffffffffu, r[F_NT], pr);
                         const float Ax = fixed_dot<DIM3>(tT0, tT1, dxv, dyv_c);
-                        if (series) {
-                            leg_series(centre_a<DIM3>(tT0, tT1, tT2, dxv, dyv_c, dvc, fmaf(dvc, dvc, d2c)),
-                                       centre_b<DIM3>(tT1, tT2, dvc), nT2, nT, sT);
-#pragma unroll
-                            for (int q = 0; q < 5; ++q) sT[q] *= p.hs_s;
-                        }
                         // seabed refraction of the transmitter leg
                         const bool trefr = REFRACT && (rfl_s[pr] & FL_T_REFR);
                         float4 tr0 = make_float4(0.f, 0.f, 0.f, 0.f), tr1 = tr0, tr2 = tr0;
@@ -180,22 +171,6 @@ __global__ void __launch_bounds__(NTHREADS, 2) adjoint_kernel(const KParams p, c
                     const float ufc = __shfl_sync(0xffffffffu, r[F_UF], pr);
                     const float phr = __shfl_sync(0xffffffffu, r[F_PH], pr);
                     const float Ax = fixed_dot<DIM3>(tRx, tRy, dxv, dyv_c);
-                    const bool use_series = series && fminf(rec[F_NT * PAIRS + pr], nR) >= p.series_rmin;
-                    float2 vser[PX / 2];   // half-sample coordinates, slots (2k, 2k + 1)
-                    if (use_series) {
-                        float c[5];
-                        leg_series(centre_a<DIM3>(tRx, tRy, tRz, dxv, dyv_c, dvc, fmaf(dvc, dvc, d2c)),
-                                   centre_b<DIM3>(tRy, tRz, dvc), nR2, nR, c);
-                        c[0] = fmaf(c[0], p.hs_s, sT[0] + ufc);
-#pragma unroll
-                        for (int q = 1; q < 5; ++q) c[q] = fmaf(c[q], p.hs_s, sT[q]);
-#pragma unroll
-                        for (int h = 0; h < PX / 4; ++h) {
-                            float2 back;
-                            series_quad(p, c, h, vser[PX / 4 + h], back);
-                            vser[PX / 4 - 1 - h] = make_float2(back.y, back.x);
-                        }
-                    }
                     // receiver motion: (R_R + d).v / c = Km + d_var v_var / c, as the forward
                     // kernel forms it; the beam test keeps the ping-time receiver vector
                     float Km = 0.f, vv = 0.f, bRx = tRx, bRy = tRy, bRz = tRz;
@@ -237,34 +212,28 @@ __global__ void __launch_bounds__(NTHREADS, 2) adjoint_kernel(const KParams p, c
                                 !beam_sees(p, fmaf(0.5f, bRx, dxv), fmaf(0.5f, bRy, dy), fmaf(0.5f, bRz, dz), rot))
                                 continue;
                         }
-                        float D = 0.f, v;                                  // v: 2 (u - floor u_ref) - 1/2
-                        if (use_series) {
-                            v = (s & 1) ? vser[s >> 1].y : vser[s >> 1].x;
-                        } else {
-                            const float d2 = fmaf(dvar[s], dvar[s], d2c);
-                            const float a = __fadd_rn(fmaf(DIM3 ? tRz : tRy, dvar[s], d2), Ax);
-                            const float sm = nR2 + a;
-                            const float rs = rsqrt_sfu(sm);
-                            D = fmaf(a, rcp_sfu(fmaf(sm, rs, nR)), dT[s]);
-                            if (REFRACT && rrefr) {
-                                if ((bmask >> s) & 1u) {
-                                    float rho = rhoR, drho = drhoR;
-                                    if (!DIM3) refr_rho(rr0, a, rho, drho);
-                                    const float db = DIM3 ? dvar[s] - r_zoff : 0.f, b = fmaxf(r_br + db, 1e-7f);
-                                    float uxi, ua;
-                                    D = refr_leg_diff(p, rr0, rr1, rr2, rho, drho, b, db, r_br, uxi, ua) + dT[s];
-                                } else {
-                                    D += rr2.w;
-                                }
+                        const float d2 = fmaf(dvar[s], dvar[s], d2c);
+                        const float a = __fadd_rn(fmaf(DIM3 ? tRz : tRy, dvar[s], d2), Ax);
+                        const float sm = nR2 + a;
+                        const float rs = rsqrt_sfu(sm);
+                        float D = fmaf(a, rcp_sfu(fmaf(sm, rs, nR)), dT[s]);
+                        if (REFRACT && rrefr) {
+                            if ((bmask >> s) & 1u) {
+                                float rho = rhoR, drho = drhoR;
+                                if (!DIM3) refr_rho(rr0, a, rho, drho);
+                                const float db = DIM3 ? dvar[s] - r_zoff : 0.f, b = fmaxf(r_br + db, 1e-7f);
+                                float uxi, ua;
+                                D = refr_leg_diff(p, rr0, rr1, rr2, rho, drho, b, db, r_br, uxi, ua) + dT[s];
+                            } else {
+                                D += rr2.w;
                             }
-                            if (p.vel) {
-                                const float eps = fmaf(dvar[s], vv, Km) * rs;         // u_R . v / c
-                                D = D * fmaf(eps, eps - 1.f, 1.f);                   // / (1 + eps)
-                            }
-                            v = fmaf(D, series ? p.hs_s : p.hs_c, ufc);
                         }
-                        // carrier phase [rad]
-                        float ph = series ? fmaf(v, p.ph_hs, fmaf(-ufc, p.ph_hs, phr)) : fmaf(D, p.wfc_c, phr);
+                        if (p.vel) {
+                            const float eps = fmaf(dvar[s], vv, Km) * rs;         // u_R . v / c
+                            D = D * fmaf(eps, eps - 1.f, 1.f);                   // / (1 + eps)
+                        }
+                        const float v = fmaf(D, p.hs_c, ufc);              // 2 (u - floor u_ref) - 1/2
+                        float ph = fmaf(D, p.wfc_c, phr);                  // carrier phase [rad]
                         // nearest integer of v = the half-sample index; g = frac(2u) - 1/2
                         const float t = __fadd_rn(v, FLOOR_MAGIC);
                         const float g = v - (t - FLOOR_MAGIC);

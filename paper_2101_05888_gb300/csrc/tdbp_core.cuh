@@ -59,7 +59,7 @@ constexpr int NTHREADS = NCONS + 32;    // + producer warp
 constexpr int PAIRS = 32;               // (ping, channel) pairs per stage
 constexpr int NSEG = 2;                 // echo-segment ring depth (stages)
 constexpr int NRS = 3;                  // record ring depth (stages)
-constexpr int NBUF = 3;                 // Farrow buffers (groups)
+constexpr int NBUF = 3;                 // Farrow buffers (groups), at most
 constexpr int GROUP = 4;                // pairs per Farrow group
 constexpr int GPS = PAIRS / GROUP;      // groups per stage
 constexpr int PX = 8;                   // pixels per consumer thread
@@ -142,7 +142,9 @@ struct KParams {
     float2 ypos[PX / 4], yneg[PX / 4], ysq[PX / 4];
     float hs_s, ph_hs, series_rmin;
     int U, npos, npos_pad, seglen, seg_align, slot_bytes;
-    int accumulate, atomic_out, skip_copies;
+    int nbuf;               // Farrow buffers of the ring (FIXED kernels: NBUF)
+    int accumulate, skip_copies;
+    size_t split_stride;    // forward: split k writes its part at image + k split_stride (0: one split)
     unsigned long long wait_ns;
 };
 
@@ -720,22 +722,15 @@ __device__ __forceinline__ float fixed_dot(float tx, float ty, float dx, float d
 // of what rounding the path to FP32 costs, which holds from series_rmin
 // (6 .. 10 m in 2D, 2 m over a 3D column) on; pairs nearer than that take the
 // exact form at every pixel.
-// Measured against an rsqrt and a rcp a pixel: 250 pings x 24 RX -> 1500 x 1101,
-// BF16: 13.53 -> 12.31 ms; 196 x 64 -> 256 x 224 x 56, FP16: 47.3 -> 43.5 ms;
-// 512 x 32 -> 4096^2, complex64: 338.6 -> 332.4 ms (there the shared-memory pipe
-// binds now, 79 % busy with 32 bytes of Farrow rows an update).
+// Measured against an rsqrt and a rcp a pixel, with the packed accumulators (16-bit
+// echoes): 250 pings x 24 RX -> 1500 x 1101: 13.53 -> 12.12 ms; 196 x 64 ->
+// 256 x 224 x 56: 47.3 -> 42.6 ms.
 // c[0] = r0 - |R| (the differential path at the line's centre), c[1 .. 4] as
-// above.  a0 = 2R.d0 + |d0|^2, b = (R + d0) . axis, n2 = |R|^2, n = |R|.  The
-// root and the quotient of c[0] take a Newton step each: the SFU's 1e-7
-// relative would cost 1e-5 rad and more over a tile's path span, and here the
-// steps are shared by PX pixels.
+// above.  a0 = 2R.d0 + |d0|^2, b = (R + d0) . axis, n2 = |R|^2, n = |R|.
 __device__ __forceinline__ void leg_series(float a0, float b, float n2, float n, float* c) {
     const float sm = n2 + a0;
     const float rs = rsqrt_sfu(sm), hr = 0.5f * rs;
-    float r0 = sm * rs;
-    r0 = fmaf(hr, fmaf(-r0, r0, sm), r0);
-    const float den = r0 + n, rc = rcp_sfu(den), q0 = a0 * rc;
-    c[0] = fmaf(rc, fmaf(-den, q0, a0), q0);
+    c[0] = a0 * rcp_sfu(fmaf(sm, rs, n));
     c[1] = b * rs;
     c[2] = hr * fmaf(-c[1], c[1], 1.f);
     const float q = c[1] * rs;
@@ -792,9 +787,12 @@ static_assert((NRS * PAIRS * NREC * 4) % 16 == 0 && (NRS * PAIRS * NREC_REFR * 4
 constexpr int NPOS_FIXED = 60;
 static_assert(NPOS_FIXED % RUN == 0, "whole expansion runs");
 
-inline size_t smem_bytes(int slot_bytes, int npos_pad, int nrec, int row_bytes) {
+// shared memory with which two CTAs fit an SM
+constexpr size_t SMEM_TWO_CTAS = 113 * 1024;
+
+inline size_t smem_bytes(int slot_bytes, int npos_pad, int nrec, int row_bytes, int nbuf) {
     return (size_t)NSEG * PAIRS * slot_bytes                   // echo segments
-           + (size_t)NBUF * GROUP * npos_pad * NH * row_bytes  // Farrow rows
+           + (size_t)nbuf * GROUP * npos_pad * NH * row_bytes  // Farrow rows
            + (size_t)NRS * PAIRS * nrec * 4                    // records
            + (size_t)NH * TAPS * NP * 4                        // coefficients
            + (size_t)NCW * 4 * 8                        // cross-warp reduction (gradient)
@@ -814,8 +812,14 @@ template <typename ET, bool DIM3, int MODE, bool BEAM, bool MOTION, bool REFRACT
 __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant__ CUtensorMap tmap, const KParams p) {
     using T = Tile<DIM3>;
     static_assert(!REFRACT || (!BEAM && !MOTION), "refraction: without the beam or receiver motion");
-    // the forward pass over straight legs takes the column series
-    constexpr bool SERIES = MODE == MODE_FORWARD && !REFRACT && !MOTION;
+    // 16-bit echoes in the forward pass over straight legs take the column series;
+    // complex64 ones keep the per-pixel legs: the kernel is bound by the shared-memory
+    // pipe there (32 bytes of rows an update), so the series gains little (64 x 32 ->
+    // 4096^2: 41.4 against 42.2 ms) for another rounding of every phase, 1.2e-5 of the image
+    constexpr bool SERIES = MODE == MODE_FORWARD && !REFRACT && !MOTION && sizeof(ET) == 4;
+    // the image accumulated as sum s cos and sum s sin, each a packed FMA an update (the
+    // rotation's cross terms are resolved once, when the tile is written)
+    constexpr bool ACC2 = MODE == MODE_FORWARD && !REFRACT;
     constexpr int KREC = REFRACT ? NREC_REFR : NREC;   // record fields
     // FP16 Farrow rows for 16-bit echoes in the forward pass; otherwise rows
     // of FP32 E0, E1 and BF16 E2, E3
@@ -830,7 +834,8 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
     unsigned char* ebuf = seg + (size_t)NSEG * PAIRS * p.slot_bytes;     // [NBUF][GROUP] Farrow rows
     const int npos_pad = FIXED ? NPOS_FIXED : p.npos_pad;
     const int ebuf_pair = npos_pad * NH * ROWB;       // positions padded to whole expansion runs
-    float* rec = reinterpret_cast<float*>(ebuf + (size_t)NBUF * GROUP * ebuf_pair);   // [NRS][PAIRS][KREC]
+    const int nbuf = FIXED ? NBUF : p.nbuf;
+    float* rec = reinterpret_cast<float*>(ebuf + (size_t)nbuf * GROUP * ebuf_pair);   // [NRS][PAIRS][KREC]
     float* coef_s = rec + NRS * PAIRS * KREC;                            // [NH][TAPS][NP]
     // every part so far has a size that is a multiple of 16 bytes (see smem_bytes)
     double* wred = reinterpret_cast<double*>(coef_s + NH * TAPS * NP);    // [NCW][4]
@@ -1039,10 +1044,9 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
         // 16-byte rows (cubic) or E2 in 8-byte rows (quadratic)
         const int plane1 = npos_pad * NH * 16;          // bytes of a pair's first plane
         const int e_off = Eq * plane1;
-        int G = 0;   // groups emitted
+        int b = 0, use = 0;   // the next group's buffer; how often the ring has gone round
         auto emit = [&](int rs, int pr0, int ng, int flags, int ss) {
-            const int b = G % NBUF;
-            if (G >= NBUF && !mbar_wait_bounded(smem_u32(&eempty[b]), ((G / NBUF) - 1) & 1, p.wait_ns)) fail();
+            if (use > 0 && !mbar_wait_bounded(smem_u32(&eempty[b]), (use - 1) & 1, p.wait_ns)) fail();
             if (SERIES) {
                 const bool exact = lane < ng && (__float_as_int(rec[(rs * PAIRS + pr0 + lane) * KREC + F_FLAGS]) & FL_EXACT);
                 if (__any_sync(0xffffffffu, exact)) flags |= GD_EXACT;
@@ -1096,7 +1100,10 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
                 gdesc[b] = make_int4(rs, pr0, ng, flags);
                 mbar_arrive(smem_u32(&efull[b]));
             }
-            ++G;
+            if (++b == nbuf) {
+                b = 0;
+                ++use;
+            }
         };
 
         bool last_cur = false, last_next = false;
@@ -1157,10 +1164,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
     // series in half samples)
     float2 dvp[SERIES ? 1 : PX / 2], d2p[SERIES ? 1 : PX / 2], dTp[SERIES ? 1 : PX / 2];
     float dvc = 0.f, d2c0 = 0.f, sT[5] = {0.f, 0.f, 0.f, 0.f, 0.f};
-    // column series: the image accumulators in two parts, sum s cos and sum s sin,
-    // each a packed FMA an update (the rotation's cross terms are resolved once,
-    // when the tile is written)
-    float2 accs[SERIES ? PX : 1];
+    float2 accs[ACC2 ? PX : 1];
 #define PXS(arr, s) (((s) & 1) ? arr[(s) >> 1].y : arr[(s) >> 1].x)
     float2 acc[PX];                       // forward: image accumulators; gradient: G(x)
     float rsum[MODE == MODE_OFFSET_GRAD ? PX : 1];
@@ -1183,9 +1187,8 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
                 PXS(dvp, s) = dvs;
                 PXS(d2p, s) = fmaf(dvs, dvs, d2c);
                 PXS(dTp, s) = 0.f;
-            } else {
-                accs[s] = make_float2(0.f, 0.f);
             }
+            if constexpr (ACC2) accs[s] = make_float2(0.f, 0.f);
             if (MODE == MODE_FORWARD) {
                 acc[s] = make_float2(0.f, 0.f);
             } else {
@@ -1286,6 +1289,17 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
         }
         named_bar_sync(BAR_CONS, NCONS);
         (void)tNT;
+    };
+
+    // image += v exp(j x) at slot s
+    auto accumulate = [&](const int s, const float2 v, const float cs, const float sn) {
+        if constexpr (ACC2) {
+            acc[s] = ffma2(v, make_float2(cs, cs), acc[s]);
+            accs[s] = ffma2(v, make_float2(sn, sn), accs[s]);
+        } else {
+            acc[s].x = fmaf(v.x, cs, fmaf(-v.y, sn, acc[s].x));
+            acc[s].y = fmaf(v.x, sn, fmaf(v.y, cs, acc[s].y));
+        }
     };
 
     // per-pixel work of one pair; MASKED: apply the beam test per pixel.  The
@@ -1417,8 +1431,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
                 const float2 e2 = *reinterpret_cast<const float2*>(erow_b + pos * 8);
                 float2 v = ffma2(e2, gg2, make_float2(e01.z, e01.w));
                 v = ffma2(v, gg2, make_float2(e01.x, e01.y));
-                acc[s].x = fmaf(v.x, cs, fmaf(-v.y, sn, acc[s].x));
-                acc[s].y = fmaf(v.x, sn, fmaf(v.y, cs, acc[s].y));
+                accumulate(s, v, cs, sn);
                 continue;
             }
             // cubic: (E2, E3) from the second plane
@@ -1430,8 +1443,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
                 float2 v = ffma2(e3, gg2, e2);
                 v = ffma2(v, gg2, e1);
                 v = ffma2(v, gg2, e0);
-                acc[s].x = fmaf(v.x, cs, fmaf(-v.y, sn, acc[s].x));
-                acc[s].y = fmaf(v.x, sn, fmaf(v.y, cs, acc[s].y));
+                accumulate(s, v, cs, sn);
             } else {
                 // value and derivative in g: b = s(g), d = ds/dg (ds/du = 2 d)
                 float2 b = e3;
@@ -1471,7 +1483,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
         }
     };
 
-    // Column-series forms of the above (forward pass, straight legs).  One
+    // Column-series forms of the above (16-bit forward pass, straight legs).  One
     // update: the row of half-sample coordinate t = v + 1.5 2^23, g = v - rint(v),
     // the carrier phase x; sum s cos(x) and sum s sin(x).
     auto update = [&](auto masked, const int s, const float tj, const float g, const float x, const bool seen,
@@ -1488,18 +1500,10 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
         }
         const float2 gg2 = make_float2(g, g);
         const float4 e01 = *reinterpret_cast<const float4*>(erow + pos * 16);
-        float2 v;
-        if constexpr (E16) {
-            const float2 e2 = *reinterpret_cast<const float2*>(erow_b + pos * 8);
-            v = ffma2(e2, gg2, make_float2(e01.z, e01.w));
-        } else {
-            const float4 e23 = *reinterpret_cast<const float4*>(erow_b + pos * 16);
-            v = ffma2(make_float2(e23.z, e23.w), gg2, make_float2(e23.x, e23.y));
-            v = ffma2(v, gg2, make_float2(e01.z, e01.w));
-        }
+        const float2 e2 = *reinterpret_cast<const float2*>(erow_b + pos * 8);
+        float2 v = ffma2(e2, gg2, make_float2(e01.z, e01.w));
         v = ffma2(v, gg2, make_float2(e01.x, e01.y));
-        acc[s] = ffma2(v, make_float2(cs, cs), acc[s]);
-        accs[SERIES ? s : 0] = ffma2(v, make_float2(sn, sn), accs[SERIES ? s : 0]);
+        accumulate(s, v, cs, sn);
     };
     // the beam test of slot s (MASKED pairs)
     auto slot_seen = [&](const int s, const float4 q0, const float* rot, uint32_t rmask_needed) {
@@ -1565,9 +1569,8 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
     bool aborted = false;
     int prev_ping = -1;
     int seq_ping = ping0, seq_ch = 0;               // candidate order (no culling)
-    for (int G = 0;; ++G) {
-        const int b = G % NBUF;
-        if (!mbar_wait_bounded(smem_u32(&efull[b]), (G / NBUF) & 1, p.wait_ns)) {
+    for (int b = 0, use = 0;;) {
+        if (!mbar_wait_bounded(smem_u32(&efull[b]), use & 1, p.wait_ns)) {
             *abort_flag = 1;
             atomicOr(p.status, DEV_TIMEOUT);
         }
@@ -1710,6 +1713,10 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
             }
         }
         warp_arrive(&eempty[b]);
+        if (++b == nbuf) {
+            b = 0;
+            ++use;
+        }
         if (gflags & GD_STAGE_END) warp_arrive(&rempty[rs]);
         if (gflags & GD_LAST) break;
     }
@@ -1724,11 +1731,9 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
         T::pixel(ct, s, lx, ly, lz);
         const int ix = tx0 + lx, iy = ty0 + ly, iz = tz0 + lz;
         if (ix >= p.nx || iy >= p.ny || iz >= p.nz) continue;
-        if constexpr (SERIES) acc[s] = make_float2(acc[s].x - accs[s].y, acc[s].y + accs[s].x);
-        float2* dst = p.image + ((size_t)iz * p.ny + iy) * p.nx + ix;
-        if (p.atomic_out) {
-            atomicAdd(dst, acc[s]);
-        } else if (p.accumulate) {
+        if constexpr (ACC2) acc[s] = make_float2(acc[s].x - accs[s].y, acc[s].y + accs[s].x);
+        float2* dst = p.image + split * p.split_stride + ((size_t)iz * p.ny + iy) * p.nx + ix;
+        if (p.accumulate) {
             const float2 o = *dst;
             *dst = make_float2(o.x + acc[s].x, o.y + acc[s].y);
         } else {
@@ -1757,8 +1762,8 @@ inline void tile_dims(int dim3, int& TXs, int& TYs, int& TZs) {
     }
 }
 
-// Fills the launch description for grid g; min_ctas: aim for at least this
-// many CTAs by splitting the pings of each tile (0 = never split); mode: the
+// Fills the launch description for grid g; slots: CTAs resident on the device,
+// for which the pings of each tile are split (0 = never split); mode: the
 // tdbp_kernel mode the launch runs (sets the Farrow row format).
 // range from which the column series holds on lines of half length ymax, for a
 // point within dmax of the tile centre: the term left out, r |C5| (y / r)^5 with
@@ -1772,7 +1777,7 @@ double series_range(sas_geometry_t h, double dmax, double ymax);
 // one a tile).
 int pick_pings_per_split(long long ntiles, int P, int C, long long slots, double overhead, long long max_blocks);
 
-int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long min_ctas, Setup& S, bool need_echo = true,
+int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long slots, Setup& S, bool need_echo = true,
             int mode = MODE_FORWARD);
 
 template <int MODE>

@@ -28,7 +28,7 @@ int pick_pings_per_split(long long ntiles, int P, int C, long long slots, double
     return best;
 }
 
-int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long min_ctas, Setup& S, bool need_echo, int mode) {
+int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long slots, Setup& S, bool need_echo, int mode) {
     int TXs, TYs, TZs;
     tile_dims(dim3, TXs, TYs, TZs);
     const double dz = dim3 ? g.dz : 0.0;
@@ -71,7 +71,15 @@ int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long min_ctas, S
     const int slot_bytes = (slot_samples * elem + 127) / 128 * 128;
     // quadratic rows for 16-bit echoes in the forward pass, else cubic rows
     const int row_bytes = (mode == MODE_FORWARD && elem == 4) ? ROW24 : ROW32;
-    const size_t smem = smem_bytes(slot_bytes, npos_pad, refract ? (int)NREC_REFR : (int)NREC, row_bytes);
+    // two Farrow buffers instead of three where that lets a second CTA onto the SM (2D
+    // complex64 pixels of 1.6 to 2.4 cm at 40 kHz: 120 -> 101 KB)
+    const int nrec = refract ? (int)NREC_REFR : (int)NREC;
+    int nbuf = NBUF;
+    if (smem_bytes(slot_bytes, npos_pad, nrec, row_bytes, 3) > SMEM_TWO_CTAS &&
+        smem_bytes(slot_bytes, npos_pad, nrec, row_bytes, 2) <= SMEM_TWO_CTAS)
+        nbuf = 2;
+    const size_t smem = smem_bytes(slot_bytes, npos_pad, nrec, row_bytes, nbuf);
+    if (smem > SMEM_TWO_CTAS) slots /= 2;    // one CTA an SM
     if (smem > 227 * 1024) {
         set_error("shared memory need %zu exceeds the per-block limit", smem);
         return SAS_ERR_UNSUPPORTED;
@@ -108,6 +116,7 @@ int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long min_ctas, S
     prm.wfc = (float)(2.0 * M_PI * h->sig.fc);
     prm.grad_scale = (float)(-2.0 / h->sig.c);
     prm.U = U; prm.npos = npos; prm.npos_pad = npos_pad; prm.seglen = seglen; prm.seg_align = align; prm.slot_bytes = slot_bytes;
+    prm.nbuf = nbuf;
     prm.rotc = h->d_rotc;
     prm.beam = h->beam_tan > 0.0;
     prm.beam_tan = (float)h->beam_tan;
@@ -164,16 +173,14 @@ int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long min_ctas, S
     prm.skip_copies = h->debug_skip_copies;
     prm.wait_ns = (unsigned long long)(h->debug_wait_ms > 0 ? h->debug_wait_ms : 4000) * 1000000ull;
     const long long ntiles = (long long)prm.tiles_x * prm.tiles_y * prm.tiles_z;
-    // small grids: split the pings of each tile over several CTAs (whole pings,
-    // so that every (tile, ping) belongs to exactly one CTA)
-    int nsplit = 1;
-    if (min_ctas > 0 && ntiles < min_ctas) {
-        nsplit = (int)std::min<long long>((min_ctas + ntiles - 1) / ntiles, h->P);
-        const long long min_pairs = 2 * PAIRS;   // keep at least two stages per CTA
-        nsplit = (int)std::max<long long>(1, std::min<long long>(nsplit, (long long)h->P * h->C / min_pairs));
-    }
-    prm.pings_per_split = (h->P + nsplit - 1) / nsplit;
-    nsplit = (h->P + prm.pings_per_split - 1) / prm.pings_per_split;
+    // split the pings of each tile over several CTAs (whole pings, so that every
+    // (tile, ping) belongs to exactly one CTA) where that shortens the last wave
+    // of CTAs: 128 pings x 4 RX -> 256^2 at 2 cm ran 320 CTAs on 152 slots (129 us a call; 84 us
+    // with 7 splits on the 304 slots of two CTAs an SM), 250 x 24 -> 1500 x 1101 in BF16 945
+    // tiles on 304 (12.1 ms; 11.0 ms in splits).  Filling the pipeline and writing a
+    // tile cost a CTA about 12 pairs' time.
+    prm.pings_per_split = slots > 0 ? pick_pings_per_split(ntiles, h->P, h->C, slots, 12.0, 16 * slots) : h->P;
+    const int nsplit = (h->P + prm.pings_per_split - 1) / prm.pings_per_split;
     prm.nsplit = nsplit;
     if (ntiles * nsplit > 0x7fffffffLL) {
         set_error("grid too large");
@@ -229,7 +236,47 @@ int launch_mode(const Setup& S, int echo_dtype, int dim3, cudaStream_t st) {
 
 template int launch_mode<MODE_FORWARD>(const Setup&, int, int, cudaStream_t);
 
+// image = (accumulate ? image : 0) + the parts in order
+__global__ void __launch_bounds__(256) sum_splits_kernel(const float2* __restrict__ parts, size_t npix, int nsplit,
+                                                         int accumulate, float2* __restrict__ image) {
+    const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
+    if (i >= npix) return;
+    float2 s = parts[i];
+    for (int k = 1; k < nsplit; ++k) s = fadd2(s, parts[k * npix + i]);
+    if (accumulate) s = fadd2(s, image[i]);
+    image[i] = s;
+}
+
 }  // namespace core
+
+// Planes for the parts of a split launch: the handle's scratch, or, while the
+// stream is being captured, stream-ordered memory (*own: to be freed after
+// use) -- a graph must not keep a pointer that a later call may replace.  nullptr:
+// no memory (the error is cleared).
+static float2* split_planes(sas_geometry_t h, size_t bytes, cudaStream_t st, bool* own) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    void* p = nullptr;
+    *own = false;
+    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
+        if (h->scratch_bytes >= bytes) return (float2*)h->d_scratch;
+        if (h->d_scratch) {
+            if (cudaStreamSynchronize(st) != cudaSuccess) return nullptr;
+            cudaFree(h->d_scratch);
+            h->d_scratch = nullptr;
+            h->scratch_bytes = 0;
+        }
+        if (cudaMalloc(&h->d_scratch, bytes) == cudaSuccess) {
+            h->scratch_bytes = bytes;
+            return (float2*)h->d_scratch;
+        }
+        h->d_scratch = nullptr;
+    } else if (cudaMallocAsync(&p, bytes, st) == cudaSuccess) {
+        *own = true;
+        return (float2*)p;
+    }
+    (void)cudaGetLastError();
+    return nullptr;
+}
 
 int launch_forward(const ForwardArgs& a) {
     core::Setup S;
@@ -237,10 +284,32 @@ int launch_forward(const ForwardArgs& a) {
     if (rc != SAS_OK) return rc;
     S.prm.image = a.image;
     S.prm.accumulate = a.accumulate;
-    S.prm.atomic_out = S.prm.nsplit > 1;
-    if (S.prm.atomic_out && !a.accumulate)
-        SAS_CUDA(cudaMemsetAsync(a.image, 0, sizeof(float2) * (size_t)a.grid.nx * a.grid.ny * S.prm.nz, a.stream));
-    return core::launch_mode<core::MODE_FORWARD>(S, a.h->echo_dtype, a.dim3, a.stream);
+    if (S.prm.nsplit == 1) return core::launch_mode<core::MODE_FORWARD>(S, a.h->echo_dtype, a.dim3, a.stream);
+    // several CTAs a tile: each writes its part to a plane of its own, added in a
+    // fixed order (with atomic additions the image depended on the CTAs' order,
+    // and it had to be cleared first); at most 16 x slots tiles' worth of planes
+    const size_t npix = (size_t)a.grid.nx * a.grid.ny * S.prm.nz;
+    bool own = false;
+    float2* parts = split_planes(a.h, sizeof(float2) * npix * S.prm.nsplit, a.stream, &own);
+    if (!parts) {   // no memory for the planes: one CTA a tile
+        rc = core::prepare(a.h, a.grid, a.dim3, 0, S);
+        if (rc != SAS_OK) return rc;
+        S.prm.image = a.image;
+        S.prm.accumulate = a.accumulate;
+        return core::launch_mode<core::MODE_FORWARD>(S, a.h->echo_dtype, a.dim3, a.stream);
+    }
+    S.prm.image = parts;
+    S.prm.split_stride = npix;
+    S.prm.accumulate = 0;
+    rc = core::launch_mode<core::MODE_FORWARD>(S, a.h->echo_dtype, a.dim3, a.stream);
+    if (rc == SAS_OK) {
+        core::sum_splits_kernel<<<(unsigned)((npix + 255) / 256), 256, 0, a.stream>>>(parts, npix, S.prm.nsplit,
+                                                                                     a.accumulate, a.image);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) rc = cuda_fail(e, "sum_splits_kernel");
+    }
+    if (own) cudaFreeAsync(parts, a.stream);
+    return rc;
 }
 
 }  // namespace sas
