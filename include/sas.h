@@ -476,18 +476,19 @@ int sas_dpc_model_delays(const sas_dpc_problem* pr, const double* d_vy, const do
  * p_z,i = p_z,0 + sum_{n<i} v_z[n] dt_n.  The normal equations are solved in
  * the equivalent variables (positions p_1 .. p_{P-1} and the last velocity),
  * where they are banded (half-bandwidth 7).  At most max_iter accepted steps;
- * stops when the loss or the step stalls (relative 1e-14).  h_loss (host,
+ * stops when the loss or the step stalls (relative 1e-14), after up to three more
+ * steps that the loss can no longer judge but that still shrink.  h_loss (host,
  * may be NULL): the final Eq. 8 value; h_iters (host, may be NULL): accepted
  * steps.  Synchronises the stream.  Errors: SAS_ERR_ARG, SAS_ERR_OOM,
  * SAS_ERR_CUDA. */
 int sas_dpc_solve(const sas_dpc_problem* pr, double* d_vy, double* d_vz, int32_t max_iter, double* h_loss,
                   int32_t* h_iters, void* cuda_stream);
 
-/* Test hook: the banded solve inside sas_dpc_solve streams its rows through
- * shared memory in chunks of 512 rows; rows (a power of two in [8, 512]) sets
- * a smaller chunk for the following calls of this process, so that small
- * problems cross chunk boundaries; rows = 0 restores 512.  The result does
- * not depend on it.  Errors: SAS_ERR_ARG. */
+/* Test hook: the solve inside sas_dpc_solve reduces its unknowns in segments of
+ * 64 rows (8 blocks of 8); rows (a power of two in [8, 512]) sets a smaller segment
+ * for the following calls of this process (rows / 8 blocks, at least 2, at most 8),
+ * so that small problems take several reductions; rows = 0 restores 64.  The
+ * result does not depend on it.  Errors: SAS_ERR_ARG. */
 int sas_debug_dpc_solve_chunk(int32_t rows);
 
 #ifdef __cplusplus

@@ -7,9 +7,10 @@
 //    position integrates all earlier velocities); in the equivalent variables
 //    q_j = p_{j+1} (j < P-1, positions of pings 1 .. P-1) and q_{P-1} = v_{P-1}
 //    every residual touches at most four consecutive nodes, so the matrix is
-//    banded (half-bandwidth 7 over the 2P sway/heave unknowns) and a banded
-//    Cholesky solves it.  The minimiser is the same (a linear change of
-//    variables); Marquardt's diagonal damping is applied in these variables.
+//    banded (half-bandwidth 7 over the 2P sway/heave unknowns): block tridiagonal
+//    in blocks of 8, solved by block cyclic reduction.  The minimiser is the
+//    same (a linear change of variables); Marquardt's diagonal damping is applied
+//    in these variables.
 #include "sas_common.cuh"
 
 #include <algorithm>
@@ -326,6 +327,14 @@ __device__ __forceinline__ V3 operator+(V3 a, V3 b) { return V3{a.x + b.x, a.y +
 __device__ __forceinline__ V3 operator-(V3 a, V3 b) { return V3{a.x - b.x, a.y - b.y, a.z - b.z}; }
 __device__ __forceinline__ V3 operator*(double s, V3 a) { return V3{s * a.x, s * a.y, s * a.z}; }
 __device__ __forceinline__ double norm(V3 a) { return sqrt(a.x * a.x + a.y * a.y + a.z * a.z); }
+// |a| and 1 / |a| from one reciprocal square root; |a| with a Newton step, so that
+// it is as accurate as sqrt
+__device__ __forceinline__ double norm_inv(V3 a, double& inv) {
+    const double s = a.x * a.x + a.y * a.y + a.z * a.z;
+    inv = rsqrt(s);
+    const double n = s * inv;
+    return fma(0.5 * inv, fma(-n, n, s), n);
+}
 
 // Position and velocity of ping i from the nodes q (sway, heave) and the known
 // along-track terms.
@@ -358,12 +367,43 @@ __global__ void dpc_lever_kernel(Prob pb, double* lev) {
     }
 }
 
-// Nodes q from velocities (positions integrated from p_0), and the along-track positions.
-__global__ void dpc_nodes_kernel(Prob pb, const double* vy, const double* vz, double* q, double* xpos) {
-    if (blockIdx.x != 0 || threadIdx.x != 0) return;
-    double x = pb.p0[0], y = pb.p0[1], z = pb.p0[2];
-    xpos[0] = x;
-    for (int i = 0; i + 1 < pb.P; ++i) {
+// Nodes q from velocities (positions integrated from p_0), and the along-track
+// positions: one block; a thread sums a run of pings, the runs' sums are added up in
+// order, and the thread walks its run again from there.
+constexpr int NODES_T = 256;
+__global__ void __launch_bounds__(NODES_T) dpc_nodes_kernel(Prob pb, const double* vy, const double* vz, double* q,
+                                                            double* xpos) {
+    __shared__ double sum[3][NODES_T];
+    const int n = pb.P - 1, per = (n + NODES_T - 1) / NODES_T;
+    const int i0 = min(n, (int)threadIdx.x * per), i1 = min(n, i0 + per);
+    double x = 0.0, y = 0.0, z = 0.0;
+    for (int i = i0; i < i1; ++i) {
+        x += pb.vx[i] * pb.dt[i];
+        y += vy[i] * pb.dt[i];
+        z += vz[i] * pb.dt[i];
+    }
+    sum[0][threadIdx.x] = x;
+    sum[1][threadIdx.x] = y;
+    sum[2][threadIdx.x] = z;
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        double s = pb.p0[threadIdx.x];
+        for (int t = 0; t < NODES_T; ++t) {
+            const double v = sum[threadIdx.x][t];
+            sum[threadIdx.x][t] = s;
+            s += v;
+        }
+    }
+    __syncthreads();
+    x = sum[0][threadIdx.x];
+    y = sum[1][threadIdx.x];
+    z = sum[2][threadIdx.x];
+    if (threadIdx.x == 0) {
+        xpos[0] = x;
+        q[2 * n] = vy[n];
+        q[2 * n + 1] = vz[n];
+    }
+    for (int i = i0; i < i1; ++i) {
         x += pb.vx[i] * pb.dt[i];
         y += vy[i] * pb.dt[i];
         z += vz[i] * pb.dt[i];
@@ -371,8 +411,6 @@ __global__ void dpc_nodes_kernel(Prob pb, const double* vy, const double* vz, do
         q[2 * i] = y;
         q[2 * i + 1] = z;
     }
-    q[2 * (pb.P - 1)] = vy[pb.P - 1];
-    q[2 * (pb.P - 1) + 1] = vz[pb.P - 1];
 }
 
 __global__ void dpc_velocities_kernel(Prob pb, const double* q, double* vy, double* vz) {
@@ -426,11 +464,21 @@ __device__ __forceinline__ Res dpc_residual(const Prob& pb, const double* q, lon
     const V3 s = v3(pb.ps + 3 * m);
     const V3 a1 = p1 + v3(l1) - s, b1 = p1 + t * v1 + v3(l1 + 3 * (c + pb.shift + 1)) - s;
     const V3 a2 = p2 + v3(l2) - s, b2 = p2 + t * v2 + v3(l2 + 3 * (c + 1)) - s;
-    const double na1 = norm(a1), nb1 = norm(b1), na2 = norm(a2), nb2 = norm(b2);
+    double na1, nb1, na2, nb2, ia1 = 0.0, ib1 = 0.0, ia2 = 0.0, ib2 = 0.0;
+    if (JAC) {
+        na1 = norm_inv(a1, ia1);
+        nb1 = norm_inv(b1, ib1);
+        na2 = norm_inv(a2, ia2);
+        nb2 = norm_inv(b2, ib2);
+    } else {
+        na1 = norm(a1);
+        nb1 = norm(b1);
+        na2 = norm(a2);
+        nb2 = norm(b2);
+    }
     Res o;
     o.r = (na1 + nb1) - (na2 + nb2) + (with_delay ? pb.c * pb.delay[m] : 0.0);
     if (JAC) {
-        const double ia1 = 1.0 / na1, ib1 = 1.0 / nb1, ia2 = 1.0 / na2, ib2 = 1.0 / nb2;
         o.dp1[0] = a1.y * ia1 + b1.y * ib1;
         o.dp1[1] = a1.z * ia1 + b1.z * ib1;
         o.dv1[0] = t * b1.y * ib1;
@@ -469,86 +517,77 @@ __device__ __forceinline__ void robust(const Prob& pb, double r, double om, doub
 // Band index of the normal matrix entry (a, b), a <= b <= a + BANDW.
 __device__ __forceinline__ size_t bidx(int a, int b) { return (size_t)a * BROW + (b - a); }
 
-// DPC part of the loss (acc[0]) and, with JAC, of the normal matrix and the
-// gradient: one block per ping pair, its (C - shift) K measurements over the
-// threads, a block reduction, one atomic per entry.
-template <bool JAC>
-__global__ void __launch_bounds__(256) dpc_assemble_kernel(Prob pb, const double* q, double* band, double* grad,
-                                                           double* acc) {
+// DPC part of the loss (acc[0]), of the normal matrix and of the gradient: one
+// block per ping pair, its (C - shift) K measurements over the threads, a block
+// reduction, one atomic per entry.  Bound by the FP64 pipe (two lanes an SM
+// and clock here): a measurement takes about 200 FP64 operations.  The 28 sums of
+// a warp are reduced by recursive halving, 31 additions a lane; a butterfly per value
+// (140) took a quarter of the kernel.
+constexpr int ASM_T = 128;
+__global__ void __launch_bounds__(ASM_T) dpc_assemble_kernel(Prob pb, const double* q, double* band, double* grad,
+                                                             double* acc) {
     const int i = blockIdx.x;   // ping pair
     const long long per = (long long)pb.nc * pb.K;
     // local unknowns: nodes i-1 (absent for i = 0), i, i+1, sway and heave each
-    constexpr int NL = 6, NT = NL * (NL + 1) / 2;
-    double cst = 0.0, g[NL] = {0, 0, 0, 0, 0, 0}, H[NT];
+    constexpr int NL = 6, NT = NL * (NL + 1) / 2, NV = 1 + NL + NT;
+    double v[32];   // loss, gradient, upper triangle (row-wise), padding
 #pragma unroll
-    for (int e = 0; e < NT; ++e) H[e] = 0.0;
+    for (int e = 0; e < 32; ++e) v[e] = 0.0;
     const double r1 = 1.0 / pb.dt[i];
     const bool last = i + 1 == pb.P - 1;
     const double r2 = last ? 1.0 : 1.0 / pb.dt[i + 1];
-    for (long long e = threadIdx.x; e < per; e += blockDim.x) {
+    for (long long e = threadIdx.x; e < per; e += ASM_T) {
         const long long m = (long long)i * per + e;
-        const Res o = dpc_residual<JAC>(pb, q, m, true);
+        const Res o = dpc_residual<true>(pb, q, m, true);
         double cm, w;
         robust(pb, o.r, pb.weight ? pb.weight[m] : 1.0, cm, w);
-        cst += cm;
-        if (JAC) {
-            double J[NL];
+        v[0] += cm;
+        double J[NL];
 #pragma unroll
-            for (int a = 0; a < 2; ++a) {
-                J[a] = i > 0 ? o.dp1[a] - o.dv1[a] * r1 : 0.0;                            // node i-1 (p_i, v_i)
-                J[2 + a] = o.dp2[a] + o.dv1[a] * r1 - (last ? 0.0 : o.dv2[a] * r2);     // node i (p_{i+1}, v_i, v_{i+1})
-                J[4 + a] = o.dv2[a] * r2;                                               // node i+1 (v_{i+1})
-            }
-            int t = 0;
+        for (int a = 0; a < 2; ++a) {
+            J[a] = i > 0 ? o.dp1[a] - o.dv1[a] * r1 : 0.0;                            // node i-1 (p_i, v_i)
+            J[2 + a] = o.dp2[a] + o.dv1[a] * r1 - (last ? 0.0 : o.dv2[a] * r2);     // node i (p_{i+1}, v_i, v_{i+1})
+            J[4 + a] = o.dv2[a] * r2;                                               // node i+1 (v_{i+1})
+        }
+        int t = 0;
 #pragma unroll
-            for (int a = 0; a < NL; ++a) {
-                g[a] = fma(w * J[a], o.r, g[a]);
+        for (int a = 0; a < NL; ++a) {
+            const double wj = w * J[a];
+            v[1 + a] = fma(wj, o.r, v[1 + a]);
 #pragma unroll
-                for (int b = a; b < NL; ++b) {
-                    H[t] = fma(w * J[a], J[b], H[t]);
-                    ++t;
-                }
+            for (int b = a; b < NL; ++b) {
+                v[1 + NL + t] = fma(wj, J[b], v[1 + NL + t]);
+                ++t;
             }
         }
     }
-    // block reduction: warps by shuffles, then across warps in shared memory
-    __shared__ double red[8][1 + NL + NT];
-    auto wsum = [&](double v) {
-#pragma unroll
-        for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(FULL, v, o);
-        return v;
-    };
+    // after the five steps lane l holds the warp's total of value l
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    cst = wsum(cst);
-    if (JAC) {
 #pragma unroll
-        for (int a = 0; a < NL; ++a) g[a] = wsum(g[a]);
+    for (int o = 16; o; o >>= 1) {
+        const bool up = lane & o;
 #pragma unroll
-        for (int e = 0; e < NT; ++e) H[e] = wsum(H[e]);
-    }
-    if (lane == 0) {
-        red[warp][0] = cst;
-        if (JAC) {
-            for (int a = 0; a < NL; ++a) red[warp][1 + a] = g[a];
-            for (int e = 0; e < NT; ++e) red[warp][1 + NL + e] = H[e];
+        for (int e = 0; e < o; ++e) {
+            const double mine = up ? v[e + o] : v[e], other = up ? v[e] : v[e + o];
+            v[e] = mine + __shfl_xor_sync(FULL, other, o);
         }
     }
+    __shared__ double red[ASM_T / 32][32];
+    red[warp][lane] = v[0];
     __syncthreads();
-    const int nw = blockDim.x >> 5;
-    const int nval = JAC ? 1 + NL + NT : 1;
-    if ((int)threadIdx.x < nval) {
-        double s = 0.0;
-        for (int w2 = 0; w2 < nw; ++w2) s += red[w2][threadIdx.x];
-        const int v = threadIdx.x;
-        if (v == 0) {
-            atomicAdd(&acc[0], s);
-        } else if (v <= NL) {
-            const int a = v - 1;
+    if (threadIdx.x < NV) {
+        const int k = threadIdx.x;
+        double sum = 0.0;
+        for (int w2 = 0; w2 < ASM_T / 32; ++w2) sum += red[w2][k];
+        if (k == 0) {
+            atomicAdd(&acc[0], sum);
+        } else if (k <= NL) {
+            const int a = k - 1;
             const int node = i - 1 + a / 2;
-            if (node >= 0) atomicAdd(&grad[2 * node + (a & 1)], s);
+            if (node >= 0) atomicAdd(&grad[2 * node + (a & 1)], sum);
         } else {
             // entry e of the upper triangle -> (a, b)
-            int e = v - 1 - NL, a = 0;
+            int e = k - 1 - NL, a = 0;
             while (e >= NL - a) {
                 e -= NL - a;
                 ++a;
@@ -557,14 +596,13 @@ __global__ void __launch_bounds__(256) dpc_assemble_kernel(Prob pb, const double
             const int na = i - 1 + a / 2, nb = i - 1 + b / 2;
             if (na >= 0 && nb >= 0) {
                 const int ga = 2 * na + (a & 1), gb = 2 * nb + (b & 1);
-                atomicAdd(&band[bidx(min(ga, gb), max(ga, gb))], s);
+                atomicAdd(&band[bidx(min(ga, gb), max(ga, gb))], sum);
             }
         }
     }
 }
 
 // Regularisers (Eqs. 6, 7): one thread per ping; loss into acc[0].
-template <bool JAC>
 __global__ void dpc_regular_kernel(Prob pb, const double* q, double* band, double* grad, double* acc) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     double cst = 0.0;
@@ -573,7 +611,7 @@ __global__ void dpc_regular_kernel(Prob pb, const double* q, double* band, doubl
         const double pz = i == 0 ? pb.p0[2] : q[2 * (i - 1) + 1];
         const double d = pz - pb.zdvl[i];
         cst += pb.lambda2 * d * d;
-        if (JAC && i > 0) {
+        if (i > 0) {
             const int u = 2 * (i - 1) + 1;
             atomicAdd(&band[bidx(u, u)], pb.lambda2);
             atomicAdd(&grad[u], pb.lambda2 * d);
@@ -613,14 +651,12 @@ __global__ void dpc_regular_kernel(Prob pb, const double* q, double* band, doubl
                 vel(i, -2.0);
                 vel(i - 1, 1.0);
                 cst += pb.lambda1 * s * s;
-                if (JAC) {
-                    for (int a = 0; a < nn; ++a) {
-                        const int ga = 2 * node[a] + comp;
-                        atomicAdd(&grad[ga], pb.lambda1 * coef[a] * s);
-                        for (int b = 0; b < nn; ++b) {
-                            const int gb = 2 * node[b] + comp;
-                            if (gb >= ga) atomicAdd(&band[bidx(ga, gb)], pb.lambda1 * coef[a] * coef[b]);
-                        }
+                for (int a = 0; a < nn; ++a) {
+                    const int ga = 2 * node[a] + comp;
+                    atomicAdd(&grad[ga], pb.lambda1 * coef[a] * s);
+                    for (int b = 0; b < nn; ++b) {
+                        const int gb = 2 * node[b] + comp;
+                        if (gb >= ga) atomicAdd(&band[bidx(ga, gb)], pb.lambda1 * coef[a] * coef[b]);
                     }
                 }
             }
@@ -638,197 +674,289 @@ __global__ void dpc_regular_kernel(Prob pb, const double* q, double* band, doubl
     }
 }
 
-// Damped banded Cholesky solve of (N + mu diag N) delta = -g and the trial
-// nodes q + delta, by one warp, right-looking: the pending entries of the next
-// BANDW + 1 rows sit in a ring in shared memory; row j's factor U(j, j + d) is
-// one multiplication by 1 / sqrt(pending diagonal) per lane, and its rank-1
-// update of the trailing 7 x 7 triangle is one FMA on each of 28 lanes, so the
-// critical path per row is one reciprocal square root and a few FP64
-// operations (no sequential dot products).  The forward substitution
-// U^T y = -g rides along (its right-hand side updated the same way); the back
-// substitution runs on one lane.  The rows of the band and of g (forward),
-// and of U and y (backward, in reverse), stream through shared memory in
-// chunks of 2^rlog rows (at most SOL_R) by asynchronous copies, the next chunk
-// in flight while the current one is used, so no global-memory latency sits
-// on the chain.  acc[1] = 1 when the factorisation fails; acc[2] = max |delta|.
-constexpr int SOL_R = 512;
-int g_sol_rlog = 9;   // chunk rows 2^9 = SOL_R; smaller through sas_debug_dpc_solve_chunk
-static_assert(BANDW == 7, "the back substitution keeps seven deltas in registers");
-constexpr size_t SOL_SMEM = sizeof(double) * 2 * SOL_R * (BROW + 1);
+// ---------------------------------------------------------------------------
+// Damped solve of (N + mu diag N) delta = -g and the trial nodes q + delta by
+// block cyclic reduction.  In blocks of BS = 8 rows the band (half-bandwidth 7)
+// is block tridiagonal, symmetric positive definite.  Eliminating a block by its
+// LDL^T leaves Schur updates of its two neighbours and couples them; eliminating
+// every second block halves the chain.  A CTA does log2(seg) such levels on a
+// segment of seg blocks (a warp per eliminated block), keeps the segment's last
+// block and hands it to the next, seg times shorter system; the last system is one
+// segment whose last block is solved directly, and the segments are substituted back
+// in the opposite order.  On a positive definite matrix this is a Cholesky
+// factorisation of a permuted matrix.
+// A chain of dependent FP64 operations bounds it (eight pivots a level): 256 blocks
+// take three reductions and three substitutions.  The band factorised row by row in
+// one warp took 2.5 ms for the same 2048 unknowns, this form about 0.06 ms.
+constexpr int BS = 8;
+constexpr int BCR_SEG = 8;                 // blocks of a segment, a power of two
+constexpr int BCR_T = 32 * (BCR_SEG / 2);  // a warp per block eliminated at a segment's first level
+constexpr int EW = 3 * BS + 1;             // stored columns of an eliminated block: L^T and 1/d, left, right, rhs
+int g_bcr_seg = BCR_SEG;                   // smaller through sas_debug_dpc_solve_chunk
+static_assert(BROW == BS, "band rows of eight diagonals");
 
-__device__ __forceinline__ void sol_copy8(double* dst, const double* src) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+// One system of nb blocks: diagonal blocks D + DL (DL: the updates the next segment's
+// eliminations make to a kept block; none for the last), couplings C (block i with
+// i + 1), right-hand sides r + rL, eliminated blocks E, solution x.
+struct BcrSystem {
+    int nb;
+    double *D, *DL, *C, *r, *rL, *E, *x;
+};
+
+// shared-memory image of a segment: slot 0 the left neighbour's updates, slot t
+// block t - 1; C[t] couples slot t with its right neighbour of the current level
+struct BcrShared {
+    double D[BCR_SEG + 1][BS * BS], C[BCR_SEG + 1][BS * BS], r[BCR_SEG + 1][BS];
+    double Y[BCR_SEG / 2][BS][2 * BS + 1];   // a warp's L^-1 [left, right, rhs]
+    double x[BCR_SEG + 1][BS];
+};
+
+// LDL^T elimination of slot t with neighbours t -+ st (one warp): lane = column of
+// [D | left | right | rhs], its eight rows in registers.  By symmetry the multiplier
+// of row j is the pivot row's entry in column j over the pivot.  Writes E
+// and Y; returns false on a pivot that is not positive.
+__device__ bool bcr_eliminate(BcrShared& S, int t, int st, double* E, double (*Y)[2 * BS + 1], double* dinv) {
+    const int lane = threadIdx.x & 31;
+    const int g = lane >> 3, c = lane & 7;
+    double a[BS];
+#pragma unroll
+    for (int k = 0; k < BS; ++k) {
+        a[k] = 0.0;
+        if (g == 0) a[k] = S.D[t][k * BS + c];
+        if (g == 1) a[k] = S.C[t - st][c * BS + k];
+        if (g == 2) a[k] = S.C[t][k * BS + c];
+        if (lane == 3 * BS) a[k] = S.r[t][k];
+    }
+    bool ok = true;
+#pragma unroll
+    for (int k = 0; k < BS; ++k) {
+        const double piv = __shfl_sync(FULL, a[k], k);
+        ok = ok && piv > 0.0;
+        dinv[k] = 1.0 / (piv > 0.0 ? piv : 1.0);
+        const double m = a[k] * dinv[k];
+#pragma unroll
+        for (int j = k + 1; j < BS; ++j) a[j] = fma(-__shfl_sync(FULL, m, j), a[k], a[j]);
+        if (lane < EW) {
+            // rows of L^T (lanes k < c < 8) with 1/d on the diagonal, and Y
+            const double e = g == 0 ? (c == k ? dinv[k] : m) : a[k];
+            E[k * EW + lane] = e;
+            if (g > 0) Y[k][lane - BS] = e;
+        }
+    }
+    __syncwarp();
+    return ok;
 }
 
-// rows [c R, min(n, c R + R)) of a [n][w] array into buf [R][w]
-__device__ __forceinline__ void sol_stage(double* buf, const double* src, int n, int w, int c, int R, int lane) {
-    const int r0 = c * R, r1 = min(n, r0 + R);
-    for (int i = lane; i < (r1 - r0) * w; i += 32) sol_copy8(buf + i, src + (size_t)r0 * w + i);
+// Schur updates of one neighbour (side 0: left, with the new coupling; 1: right)
+__device__ void bcr_update(BcrShared& S, int t, int st, int side, const double (*Y)[2 * BS + 1], const double* dinv) {
+    const int lane = threadIdx.x & 31;
+    const int nbr = side ? t + st : t - st, off = side ? BS : 0;
+    // entries: D (64), rhs (8), and for the left neighbour the coupling (64)
+    for (int o = lane; o < (side ? 72 : 136); o += 32) {
+        const int row = o < 64 ? o >> 3 : (o < 72 ? o - 64 : (o - 72) >> 3);
+        const int col = o < 64 ? off + (o & 7) : (o < 72 ? 2 * BS : BS + ((o - 72) & 7));
+        double sum = 0.0;
+#pragma unroll
+        for (int k = 0; k < BS; ++k) sum = fma(Y[k][off + row] * dinv[k], Y[k][col], sum);
+        if (o < 64)
+            S.D[nbr][o] -= sum;
+        else if (o < 72)
+            S.r[nbr][row] -= sum;
+        else
+            S.C[nbr][o - 72] = -sum;
+    }
 }
 
-__global__ void __launch_bounds__(32) dpc_solve_kernel(int n, const double* band, const double* grad, double mu,
-                                                       double* work, const double* q, double* q_try, double* acc,
-                                                       int rlog) {
-    extern __shared__ __align__(16) double sol_sm[];
-    double* bbuf = sol_sm;                          // [2][SOL_R][BROW]: band rows, then U rows
-    double* gbuf = sol_sm + 2 * SOL_R * BROW;       // [2][SOL_R]: g, then y
-    __shared__ double Pm[BROW][BROW];   // Pm[r % BROW][d] = pending A(r, r + d), rows j .. j + BANDW
-    __shared__ double tv[BROW];         // pending right-hand side of those rows
-    const int lane = threadIdx.x;
-    double* U = work;                   // [n][BROW], the diagonal stored inverted
-    double* y = work + (size_t)n * BROW;
-    const int R = 1 << rlog;            // chunk rows, 8 .. SOL_R; buffers keep the SOL_R stride
-    const int nch = (n + R - 1) / R;
-    auto commit = [] { asm volatile("cp.async.commit_group;" ::: "memory"); };
-    auto wait1 = [] { asm volatile("cp.async.wait_group 1;" ::: "memory"); };
-    auto wait0 = [] { asm volatile("cp.async.wait_group 0;" ::: "memory"); };
-    auto stage_fwd = [&](int c) {
-        sol_stage(bbuf + (c & 1) * SOL_R * BROW, band, n, BROW, c, R, lane);
-        sol_stage(gbuf + (c & 1) * SOL_R, grad, n, 1, c, R, lane);
-        commit();
-    };
-    // lane -> entry (j + ta, j + tb) of the trailing triangle, 1 <= ta <= tb <= BANDW
-    int ta = 1, e = lane;
-    while (ta <= BANDW && e >= BANDW - ta + 1) {
-        e -= BANDW - ta + 1;
-        ++ta;
+// x of slot t from its neighbours' (one warp): D L^T x = Y_rhs - Y_left x_left - Y_right x_right
+__device__ void bcr_substitute(BcrShared& S, int t, int st, const double* E) {
+    const int lane = threadIdx.x & 31, k = lane >> 2, part = lane & 3;
+    double z = 0.0;
+#pragma unroll
+    for (int u = 0; u < BS / 2; ++u) {      // four lanes a row, four of its 16 products each
+        const int c = part * (BS / 2) + u;
+        const double xv = c < BS ? S.x[t - st][c] : S.x[t + st][c - BS];
+        z = fma(E[k * EW + BS + c], xv, z);
     }
-    const int tb = ta + e;
-    const bool upd = lane < BANDW * (BANDW + 1) / 2;
-    // row r of the damped matrix and of -g (lanes 0 .. BANDW; zero past the end),
-    // from its staged chunk
-    auto fetch = [&](int r, double& a, double& t) {
-        a = 0.0;
-        t = 0.0;
-        if (lane <= BANDW && r < n && r + lane < n) {
-            const int c = r >> rlog, i = r & (R - 1);
-            a = bbuf[((c & 1) * SOL_R + i) * BROW + lane];
-            if (lane == 0) {
-                a += mu * (a + 1e-12);   // Marquardt's scaling, Levenberg's floor
-                t = -gbuf[(c & 1) * SOL_R + i];
-            }
-        }
-    };
-    if (lane == 0) acc[1] = 0.0;
-    stage_fwd(0);
-    if (nch > 1) {
-        stage_fwd(1);
-        wait1();
-    } else {
-        wait0();
+    z += __shfl_xor_sync(FULL, z, 1);
+    z += __shfl_xor_sync(FULL, z, 2);
+    z = E[k * EW + k] * (E[k * EW + 3 * BS] - z);
+#pragma unroll
+    for (int j = BS - 1; j > 0; --j) {
+        const double xj = __shfl_sync(FULL, z, 4 * j);
+        if (k < j) z = fma(-E[k * EW + j], xj, z);
     }
+    if (part == 0) S.x[t][k] = z;
     __syncwarp();
-    for (int r = 0; r < BROW; ++r) {
-        double a, t;
-        fetch(r, a, t);
-        if (lane <= BANDW) Pm[r][lane] = a;
-        if (lane == 0) tv[r] = t;
+}
+
+// Substitution within a segment whose outer solutions are in S.x[0] and S.x[seg];
+// the segment's solutions go to sys.x, at the first system also to the trial nodes
+// (first: q_try = q + x over n rows, acc[2] = max |x|)
+__device__ void bcr_backward(BcrShared& S, const BcrSystem& sys, int seg, int s, int n, const double* q, double* q_try,
+                             double* acc) {
+    const int warp = threadIdx.x >> 5;
+    for (int st = seg / 2; st >= 1; st >>= 1) {
+        const int t = st * (2 * warp + 1);
+        if (t < seg) bcr_substitute(S, t, st, sys.E + (size_t)(s * seg + t - 1) * BS * EW);
+        __syncthreads();
     }
-    __syncwarp();
-    for (int j = 0; j < n; ++j) {
-        const int rn = j + BROW;
-        if (rn < n && (rn & (R - 1)) == 0) {
-            // the fetches move to chunk rn / R: chunk rn / R - 1 is done with,
-            // its buffer takes chunk rn / R + 1
-            const int c = rn >> rlog;
-            __syncwarp();
-            if (c + 1 < nch) {
-                stage_fwd(c + 1);
-                wait1();
-            } else {
-                wait0();
-            }
-            __syncwarp();
-        }
-        double an, tn;
-        fetch(rn, an, tn);
-        const int sj = j % BROW;
-        const double djj = Pm[sj][0];
-        if (!(djj > 0.0)) {
-            if (lane == 0) acc[1] = 1.0;
-            wait0();
-            return;
-        }
-        const double inv = rsqrt(djj);
-        double u = 0.0;
-        if (lane <= BANDW && j + lane < n) {
-            u = lane == 0 ? djj * inv : Pm[sj][lane] * inv;
-            U[(size_t)j * BROW + lane] = lane == 0 ? inv : u;
-        }
-        const double yj = tv[sj] * inv;
-        if (lane == 0) y[j] = yj;
-        const double ua = __shfl_sync(FULL, u, ta & 31), ub = __shfl_sync(FULL, u, tb & 31);
-        __syncwarp();
-        if (upd && j + tb < n) Pm[(j + ta) % BROW][tb - ta] -= ua * ub;
-        if (lane >= 1 && lane <= BANDW && j + lane < n) tv[(j + lane) % BROW] -= u * yj;
-        // row j's slot takes row j + BROW (untouched by rows <= j: it lies beyond their band)
-        if (lane <= BANDW) Pm[sj][lane] = an;
-        if (lane == 0) tv[sj] = tn;
-        __syncwarp();
-    }
-    wait0();
-    // U delta = y, rows n - 1 .. 0, U and y streamed back in reverse chunks
-    __threadfence_block();
-    __syncwarp();
-    auto stage_bwd = [&](int c) {
-        sol_stage(bbuf + (c & 1) * SOL_R * BROW, U, n, BROW, c, R, lane);
-        sol_stage(gbuf + (c & 1) * SOL_R, y, n, 1, c, R, lane);
-        commit();
-    };
-    stage_bwd(nch - 1);
-    if (nch > 1) {
-        stage_bwd(nch - 2);
-        wait1();
-    } else {
-        wait0();
-    }
-    __syncwarp();
-    // delta of rows j + 1 .. j + 7 in registers; the terms of rows j + 2 ..
-    // j + 7 are summed before delta_{j+1} is known, so one FMA and one
-    // multiplication per row are on the dependent chain
-    double d1 = 0.0, d2 = 0.0, d3 = 0.0, d4 = 0.0, d5 = 0.0, d6 = 0.0, d7 = 0.0;
     double dmax = 0.0;
-    for (int j = n - 1; j >= 0; --j) {
-        const int c = j >> rlog, i = j & (R - 1);
-        if (i == R - 1 && c < nch - 1) {
-            // entering chunk c from above: chunk c + 1 is done with, its buffer
-            // takes chunk c - 1
-            __syncwarp();
-            if (c >= 1) {
-                stage_bwd(c - 1);
-                wait1();
-            } else {
-                wait0();
-            }
-            __syncwarp();
-        }
-        if (lane == 0) {
-            // entries past row n - 1 were never written: only j + d < n is read
-            const double* Ur = bbuf + ((c & 1) * SOL_R + i) * BROW;
-            double s = gbuf[(c & 1) * SOL_R + i];
-            if (j + 7 < n) s -= Ur[7] * d7;
-            if (j + 6 < n) s -= Ur[6] * d6;
-            if (j + 5 < n) s -= Ur[5] * d5;
-            if (j + 4 < n) s -= Ur[4] * d4;
-            if (j + 3 < n) s -= Ur[3] * d3;
-            if (j + 2 < n) s -= Ur[2] * d2;
-            if (j + 1 < n) s -= Ur[1] * d1;
-            const double dj = s * Ur[0];
-            d7 = d6;
-            d6 = d5;
-            d5 = d4;
-            d4 = d3;
-            d3 = d2;
-            d2 = d1;
-            d1 = dj;
-            y[j] = dj;
-            dmax = fmax(dmax, fabs(dj));
-            q_try[j] = q[j] + dj;
+    for (int e = threadIdx.x; e < seg * BS; e += blockDim.x) {
+        const int i = s * seg + e / BS;
+        if (i >= sys.nb) continue;
+        const double x = S.x[1 + e / BS][e % BS];
+        sys.x[(size_t)i * BS + e % BS] = x;
+        const int row = i * BS + e % BS;
+        if (q_try && row < n) {
+            q_try[row] = q[row] + x;
+            dmax = fmax(dmax, fabs(x));
         }
     }
-    wait0();
-    if (lane == 0) acc[2] = dmax;
+    // the bits of non-negative doubles order like their values
+    if (q_try) atomicMax(reinterpret_cast<unsigned long long*>(&acc[2]), (unsigned long long)__double_as_longlong(dmax));
+}
+
+// Reduces segment blockIdx.x of `sys` to its last block, block blockIdx.x of `next`.
+// band != nullptr: sys is the first system, read from the band (n rows, damped; rows past n are
+// unit rows).  A single segment is solved and substituted at once.
+__global__ void __launch_bounds__(BCR_T) bcr_reduce_kernel(BcrSystem sys, BcrSystem next, int seg, int n,
+                                                           const double* band, const double* grad, double mu,
+                                                           const double* q, double* q_try, double* acc) {
+    __shared__ BcrShared S;
+    const int s = blockIdx.x, i0 = s * seg, warp = threadIdx.x >> 5;
+    for (int e = threadIdx.x; e < (seg + 1) * BS * BS; e += blockDim.x) {
+        const int t = e / (BS * BS), k = (e / BS) % BS, c = e % BS, i = i0 + t - 1;
+        double d = 0.0, cp = 0.0;
+        if (band) {
+            const int ra = i * BS + k, rb = i * BS + c, lo = min(ra, rb), hi = max(ra, rb);
+            if (i >= 0) {
+                if (hi < n && t > 0) d = band[bidx(lo, hi)];
+                if (t > 0 && k == c) d = ra < n ? d + mu * (d + 1e-12) : 1.0;   // Marquardt's scaling, Levenberg's floor
+                // row k of block i with row c of block i + 1: BS + c - k diagonals off
+                if (c < k && (i + 1) * BS + c < n) cp = band[bidx(ra, (i + 1) * BS + c)];
+            }
+        } else if (i >= 0 && i < sys.nb) {
+            const size_t o = (size_t)i * BS * BS + k * BS + c;
+            if (t > 0) d = sys.D[o] + (i + 1 < sys.nb ? sys.DL[o] : 0.0);
+            if (i + 1 < sys.nb) cp = sys.C[o];
+        } else if (t > 0 && k == c) {
+            d = 1.0;
+        }
+        S.D[t][e % (BS * BS)] = d;
+        S.C[t][e % (BS * BS)] = t < seg ? cp : 0.0;
+    }
+    for (int e = threadIdx.x; e < (seg + 1) * BS; e += blockDim.x) {
+        const int t = e / BS, k = e % BS, i = i0 + t - 1;
+        double r = 0.0;
+        if (t > 0) {
+            if (band)
+                r = i * BS + k < n ? -grad[i * BS + k] : 0.0;
+            else if (i < sys.nb)
+                r = sys.r[(size_t)i * BS + k] + (i + 1 < sys.nb ? sys.rL[(size_t)i * BS + k] : 0.0);
+        }
+        S.r[t][k] = r;
+    }
+    __syncthreads();
+    bool ok = true;
+    for (int st = 1; st < seg; st <<= 1) {
+        const int t = st * (2 * warp + 1);
+        double dinv[BS];
+        if (t < seg) {
+            ok = bcr_eliminate(S, t, st, sys.E + (size_t)(i0 + t - 1) * BS * EW, S.Y[warp], dinv) && ok;
+            bcr_update(S, t, st, 0, S.Y[warp], dinv);
+        }
+        __syncthreads();   // a kept block is one warp's left and another's right neighbour
+        if (t < seg) bcr_update(S, t, st, 1, S.Y[warp], dinv);
+        __syncthreads();
+    }
+    if (gridDim.x > 1) {
+        for (int e = threadIdx.x; e < BS * BS; e += blockDim.x) {
+            next.D[(size_t)s * BS * BS + e] = S.D[seg][e];
+            if (s > 0) {
+                next.DL[(size_t)(s - 1) * BS * BS + e] = S.D[0][e];
+                next.C[(size_t)(s - 1) * BS * BS + e] = S.C[0][e];
+            }
+        }
+        if (threadIdx.x < BS) {
+            next.r[(size_t)s * BS + threadIdx.x] = S.r[seg][threadIdx.x];
+            if (s > 0) next.rL[(size_t)(s - 1) * BS + threadIdx.x] = S.r[0][threadIdx.x];
+        }
+    } else {
+        // the last block by itself (its neighbours: none)
+        if (warp == 0) {
+            double dinv[BS];
+            for (int e = threadIdx.x; e < BS * BS; e += 32) S.C[seg][e] = S.C[0][e] = 0.0;
+            if (threadIdx.x < BS) S.x[0][threadIdx.x] = 0.0;
+            __syncwarp();
+            double* E = sys.E + (size_t)(i0 + seg - 1) * BS * EW;
+            ok = bcr_eliminate(S, seg, seg, E, S.Y[0], dinv) && ok;
+            if (threadIdx.x == 0) {
+                double x[BS];
+                for (int k = BS - 1; k >= 0; --k) {
+                    double z = dinv[k] * S.Y[0][k][2 * BS];
+                    for (int j = k + 1; j < BS; ++j) z = fma(-E[k * EW + j], x[j], z);
+                    x[k] = z;
+                    S.x[seg][k] = z;
+                }
+            }
+        }
+        __syncthreads();
+        bcr_backward(S, sys, seg, s, n, q, q_try, acc);
+    }
+    if (!ok && (threadIdx.x & 31) == 0) acc[1] = 1.0;
+}
+
+// Substitutes segment blockIdx.x of `sys` from the solution of `next`.
+__global__ void __launch_bounds__(BCR_T) bcr_backward_kernel(BcrSystem sys, BcrSystem next, int seg, int n,
+                                                             const double* q, double* q_try, double* acc) {
+    __shared__ BcrShared S;
+    const int s = blockIdx.x;
+    if (threadIdx.x < BS) {
+        S.x[0][threadIdx.x] = s > 0 ? next.x[(size_t)(s - 1) * BS + threadIdx.x] : 0.0;
+        S.x[seg][threadIdx.x] = next.x[(size_t)s * BS + threadIdx.x];
+    }
+    __syncthreads();
+    bcr_backward(S, sys, seg, s, n, q, q_try, acc);
+}
+
+// Scratch doubles of all systems of an n-row solve (blocks padded to whole segments).
+size_t bcr_doubles(int n, int seg) {
+    size_t total = 0;
+    for (int nb = (n + BS - 1) / BS;; nb = (nb + seg - 1) / seg) {
+        const size_t pad = (size_t)((nb + seg - 1) / seg) * seg;
+        total += pad * (3 * BS * BS + 2 * BS + BS * EW + BS);
+        if (nb <= seg) return total;
+    }
+}
+
+cudaError_t bcr_solve(int n, int seg, const double* band, const double* grad, double mu, double* work, const double* q,
+                      double* q_try, double* acc, cudaStream_t st) {
+    BcrSystem sys[32];
+    int ns = 0;
+    for (int nb = (n + BS - 1) / BS;; nb = (nb + seg - 1) / seg) {
+        const size_t pad = (size_t)((nb + seg - 1) / seg) * seg;
+        BcrSystem& y = sys[ns++];
+        y.nb = nb;
+        y.D = work;
+        y.DL = y.D + pad * BS * BS;
+        y.C = y.DL + pad * BS * BS;
+        y.r = y.C + pad * BS * BS;
+        y.rL = y.r + pad * BS;
+        y.E = y.rL + pad * BS;
+        y.x = y.E + pad * BS * EW;
+        work = y.x + pad * BS;
+        if (nb <= seg) break;
+    }
+    for (int k = 0; k < ns; ++k) {
+        const int nseg = (sys[k].nb + seg - 1) / seg;
+        bcr_reduce_kernel<<<nseg, BCR_T, 0, st>>>(sys[k], k + 1 < ns ? sys[k + 1] : BcrSystem{}, seg, n,
+                                                  k == 0 ? band : nullptr, grad, mu, q, k == 0 ? q_try : nullptr, acc);
+    }
+    for (int k = ns - 2; k >= 0; --k) {
+        const int nseg = (sys[k].nb + seg - 1) / seg;
+        bcr_backward_kernel<<<nseg, BCR_T, 0, st>>>(sys[k], sys[k + 1], seg, n, q, k == 0 ? q_try : nullptr, acc);
+    }
+    return cudaGetLastError();
 }
 
 inline int blocks_for(long long n, int t) { return (int)((n + t - 1) / t); }
@@ -890,7 +1018,7 @@ struct Scratch {
 // Rotated levers, along-track positions and nodes from the velocities.
 int setup(Prob& pb, Scratch& S, const double* vy, const double* vz, cudaStream_t st) {
     dpc_lever_kernel<<<blocks_for(pb.P, 128), 128, 0, st>>>(pb, S.lev);
-    dpc_nodes_kernel<<<1, 1, 0, st>>>(pb, vy, vz, S.q, S.xpos);
+    dpc_nodes_kernel<<<1, NODES_T, 0, st>>>(pb, vy, vz, S.q, S.xpos);
     SAS_CUDA(cudaGetLastError());
     pb.lev = S.lev;
     pb.xpos = S.xpos;
@@ -994,66 +1122,60 @@ extern "C" int sas_dpc_solve(const sas_dpc_problem* pr, double* d_vy, double* d_
     cudaStream_t st = (cudaStream_t)stream;
     Prob pb = make_prob(pr);
     const int n = 2 * pb.P;
-    // scratch after the nodes: q_try [n], band [n][BROW], grad [n], work [n][BROW + 1], acc [4]
-    const size_t extra = (size_t)n + (size_t)n * BROW + n + (size_t)n * (BROW + 1) + 4;
+    // scratch after the nodes: q_try [n], acc [4], two sets of band [n][BROW] and grad [n],
+    // the solver's systems
+    const int seg = g_bcr_seg;
+    const size_t nset = (size_t)n * (BROW + 1);
     Scratch S;
-    rc = S.alloc(pb, extra, st);
+    rc = S.alloc(pb, (size_t)n + 4 + 2 * nset + bcr_doubles(n, seg), st);
     if (rc != SAS_OK) return rc;
     double* q_try = S.q + n;
-    double* band = q_try + n;
-    double* grad = band + (size_t)n * BROW;
-    double* work = grad + n;
-    double* acc = work + (size_t)n * (BROW + 1);
-    double hacc[4];
+    double* acc = q_try + n;
+    double* cur = acc + 4;             // normal matrix and gradient at S.q
+    double* nxt = cur + nset;          // at q_try
+    double* work = nxt + nset;
+    double hacc[4] = {0.0, 0.0, 0.0, 0.0};
     int iters = 0;
     double cost = 0.0;
     auto fail = [&](cudaError_t e, const char* what) {
         rc = cuda_fail(e, what);
         return rc;
     };
-    auto loss_at = [&](const double* qq, double& out) -> int {
-        cudaError_t e = cudaMemsetAsync(acc, 0, sizeof(double), st);
-        if (e != cudaSuccess) return fail(e, "memset");
-        dpc_assemble_kernel<false><<<pb.P - 1, 256, 0, st>>>(pb, qq, band, grad, acc);
-        dpc_regular_kernel<false><<<blocks_for(pb.P, 128), 128, 0, st>>>(pb, qq, band, grad, acc);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) return fail(e, "dpc loss");
-        e = cudaMemcpyAsync(hacc, acc, sizeof(double), cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        if (e != cudaSuccess) return fail(e, "dpc loss readback");
-        out = hacc[0];
-        return SAS_OK;
+    // loss, normal matrix and gradient at qq (the loss into acc[0])
+    auto linearise = [&](const double* qq, double* set) -> cudaError_t {
+        cudaError_t e = cudaMemsetAsync(set, 0, sizeof(double) * nset, st);
+        if (e != cudaSuccess) return e;
+        double *band = set, *grad = set + (size_t)n * BROW;
+        dpc_assemble_kernel<<<pb.P - 1, ASM_T, 0, st>>>(pb, qq, band, grad, acc);
+        dpc_regular_kernel<<<blocks_for(pb.P, 128), 128, 0, st>>>(pb, qq, band, grad, acc);
+        return cudaGetLastError();
+    };
+    auto read_acc = [&]() -> cudaError_t {
+        cudaError_t e = cudaMemcpyAsync(hacc, acc, 3 * sizeof(double), cudaMemcpyDeviceToHost, st);
+        return e == cudaSuccess ? cudaStreamSynchronize(st) : e;
     };
     rc = setup(pb, S, d_vy, d_vz, st);
     if (rc == SAS_OK) {
-        const cudaError_t ea =
-            cudaFuncSetAttribute(dpc_solve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SOL_SMEM);
-        if (ea != cudaSuccess) fail(ea, "dpc solve attribute");
+        cudaError_t e = cudaMemsetAsync(acc, 0, 4 * sizeof(double), st);
+        if (e == cudaSuccess) e = linearise(S.q, cur);
+        if (e == cudaSuccess) e = read_acc();
+        if (e != cudaSuccess)
+            fail(e, "dpc loss");
+        else
+            cost = hacc[0];
     }
-    if (rc == SAS_OK) rc = loss_at(S.q, cost);
-    double mu = 1e-3;
+    double mu = 1e-3, last_step = 0.0;
+    int polish = 0;   // steps taken after the loss stalled
     for (int it = 0; rc == SAS_OK && it < max_iter; ++it) {
-        // normal equations at the current nodes
-        cudaError_t e = cudaMemsetAsync(band, 0, sizeof(double) * ((size_t)n * BROW + n), st);
-        if (e != cudaSuccess) {
-            fail(e, "memset");
-            break;
-        }
-        e = cudaMemsetAsync(acc, 0, sizeof(double), st);
-        dpc_assemble_kernel<true><<<pb.P - 1, 256, 0, st>>>(pb, S.q, band, grad, acc);
-        dpc_regular_kernel<true><<<blocks_for(pb.P, 128), 128, 0, st>>>(pb, S.q, band, grad, acc);
-        e = cudaGetLastError();
-        if (e != cudaSuccess) {
-            fail(e, "dpc assemble");
-            break;
-        }
         bool accepted = false, stalled = false;
-        double trial = cost;
+        double trial = cost, step = 0.0;
         for (int tries = 0; tries < 40 && rc == SAS_OK; ++tries) {
-            dpc_solve_kernel<<<1, 32, SOL_SMEM, st>>>(n, band, grad, mu, work, S.q, q_try, acc, g_sol_rlog);
-            e = cudaGetLastError();
-            if (e == cudaSuccess) e = cudaMemcpyAsync(hacc, acc, 4 * sizeof(double), cudaMemcpyDeviceToHost, st);
-            if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+            // the step, and the normal equations at the trial point with its loss (needed
+            // next when it is accepted, as it nearly always is): one read-back a trial
+            cudaError_t e = cudaMemsetAsync(acc, 0, 4 * sizeof(double), st);
+            if (e == cudaSuccess) e = bcr_solve(n, seg, cur, cur + (size_t)n * BROW, mu, work, S.q, q_try, acc, st);
+            if (e == cudaSuccess) e = linearise(q_try, nxt);
+            if (e == cudaSuccess) e = read_acc();
             if (e != cudaSuccess) {
                 fail(e, "dpc solve");
                 break;
@@ -1062,21 +1184,31 @@ extern "C" int sas_dpc_solve(const sas_dpc_problem* pr, double* d_vy, double* d_
                 mu *= 10.0;
                 continue;
             }
-            const double step = hacc[2];
-            if (loss_at(q_try, trial) != SAS_OK) break;
-            if (trial <= cost) {
+            step = hacc[2];
+            trial = hacc[0];
+            // a rise within the loss's rounding is no reason to reject a step: it would be
+            // repeated with more damping, tens of times
+            if (trial - cost <= (polish ? 1e-13 : 1e-14) * cost) {
                 std::swap(S.q, q_try);
+                std::swap(cur, nxt);
                 accepted = true;
                 stalled = (cost - trial) <= 1e-14 * cost || step == 0.0;
                 mu = std::max(mu / 3.0, 1e-15);
                 break;
             }
+            if (polish) break;
             mu *= 4.0;
         }
         if (rc != SAS_OK || !accepted) break;
         ++iters;
         cost = trial;
-        if (stalled) break;
+        // once the loss cannot tell any more (its rounding hides 1e-7 of the weakly determined
+        // directions), up to three more steps while they keep shrinking
+        if (stalled || polish) {
+            if (step == 0.0 || polish == 3 || (polish && step > 0.5 * last_step)) break;
+            ++polish;
+            last_step = step;
+        }
     }
     if (rc == SAS_OK) {
         dpc_velocities_kernel<<<blocks_for(pb.P, 128), 128, 0, st>>>(pb, S.q, d_vy, d_vz);
@@ -1094,13 +1226,11 @@ extern "C" int sas_dpc_solve(const sas_dpc_problem* pr, double* d_vy, double* d_
 }
 
 extern "C" int sas_debug_dpc_solve_chunk(int32_t rows) {
-    if (rows == 0) rows = SOL_R;
-    int lg = 3;
-    while ((1 << lg) < rows && lg < 9) ++lg;
-    if (rows < 8 || rows > SOL_R || (1 << lg) != rows) {
+    if (rows == 0) rows = 512;
+    if (rows < 8 || rows > 512 || (rows & (rows - 1)) != 0) {
         set_error("sas_debug_dpc_solve_chunk: rows must be 0 or a power of two in [8, 512]");
         return SAS_ERR_ARG;
     }
-    g_sol_rlog = lg;
+    g_bcr_seg = std::min(BCR_SEG, std::max(2, rows / BS));
     return SAS_OK;
 }
