@@ -200,43 +200,43 @@ __device__ double i0_series(double x) {
     return sum;
 }
 
-// weights of all TAPS taps at fraction f (kind 0: Kaiser-sinc; 1: table, linear in f)
-__device__ void interp_weights(int kind, double beta, int table_n, const float* table, double f, double* w) {
+// weight of tap m at fraction f (kind 0: Kaiser-sinc, not yet normalised; 1: table,
+// linear in f)
+__device__ double interp_weight(int kind, double beta, int table_n, const float* table, double f, int m) {
     if (kind == SAS_INTERP_KAISER_SINC) {
-        const double h = 0.5 * TAPS, i0b = i0_series(beta);
-        double sum = 0.0;
-        for (int m = 0; m < TAPS; ++m) {
-            const double d = f - (double)(m - TAPS / 2 + 1);
-            double v = 0.0;
-            if (fabs(d) < h) {
-                const double s2 = 1.0 - (d / h) * (d / h);
-                const double sinc = (d == 0.0) ? 1.0 : sin(M_PI * d) / (M_PI * d);
-                v = sinc * i0_series(beta * sqrt(s2)) / i0b;
-            }
-            w[m] = v;
-            sum += v;
-        }
-        for (int m = 0; m < TAPS; ++m) w[m] /= sum;
-    } else {
-        double x = f * table_n;
-        int j = (int)floor(x);
-        if (j < 0) j = 0;
-        if (j > table_n - 1) j = table_n - 1;
-        const double r = x - j;
-        for (int m = 0; m < TAPS; ++m)
-            w[m] = (1.0 - r) * (double)table[(size_t)j * TAPS + m] + r * (double)table[(size_t)(j + 1) * TAPS + m];
+        const double h = 0.5 * TAPS, d = f - (double)(m - TAPS / 2 + 1);
+        if (!(fabs(d) < h)) return 0.0;
+        const double s2 = 1.0 - (d / h) * (d / h);
+        const double sinc = (d == 0.0) ? 1.0 : sin(M_PI * d) / (M_PI * d);
+        return sinc * i0_series(beta * sqrt(s2)) / i0_series(beta);
     }
+    double x = f * table_n;
+    int j = (int)floor(x);
+    if (j < 0) j = 0;
+    if (j > table_n - 1) j = table_n - 1;
+    const double r = x - j;
+    return (1.0 - r) * (double)table[(size_t)j * TAPS + m] + r * (double)table[(size_t)(j + 1) * TAPS + m];
+}
+__device__ void normalise_weights(double* w) {
+    double sum = 0.0;
+    for (int m = 0; m < TAPS; ++m) sum += w[m];
+    for (int m = 0; m < TAPS; ++m) w[m] /= sum;
+}
+// weights of all TAPS taps at fraction f
+__device__ void interp_weights(int kind, double beta, int table_n, const float* table, double f, double* w) {
+    for (int m = 0; m < TAPS; ++m) w[m] = interp_weight(kind, beta, table_n, table, f, m);
+    if (kind == SAS_INTERP_KAISER_SINC) normalise_weights(w);
 }
 
 // Monomial coefficients in g of tap t's weight on half h, from its values at
-// the N Chebyshev nodes of the half (FP64, not rounded).
+// the N Chebyshev nodes of the half (FP64, not rounded); ck[k N + j] = T_k at node j.
 template <int N>
-__device__ void fit_half_tap(const double (*node_w)[TAPS], int t, double mono_g[N]) {
+__device__ void fit_half_tap(const double (*node_w)[TAPS], int t, const double* ck, double mono_g[N]) {
     // Chebyshev coefficients a_k = (2/N) sum_j y_j T_k(x_j), a_0 halved
     double a[N];
     for (int k = 0; k < N; ++k) {
         double s = 0.0;
-        for (int j = 0; j < N; ++j) s += node_w[j][t] * cos(M_PI * k * (j + 0.5) / N);
+        for (int j = 0; j < N; ++j) s += node_w[j][t] * ck[k * N + j];
         a[k] = 2.0 * s / N;
     }
     a[0] *= 0.5;
@@ -281,32 +281,52 @@ __device__ double form_error(int kind, double beta, int table_n, const float* ta
     return e;
 }
 
-__global__ void fit_interp_kernel(int kind, double beta, int table_n, const float* table, FarrowCoef* out,
-                                  double* err) {
-    __shared__ double node_c[NH][NP][TAPS], node_q[NH][NQ][TAPS];
+// One block.  A thread evaluates one tap at one node (FP64 Bessel series, sines and
+// roots have long latencies on this part: a thread per node took 60 us for
+// its eight taps), then a thread per node normalises and a thread per (half, tap)
+// converts.  err != nullptr: also the largest deviation from the definition over 2049
+// fractions (2.9 ms; only the evaluation entry points ask for it -- every new handle's
+// first image used to wait for it).
+__global__ void __launch_bounds__(128) fit_interp_kernel(int kind, double beta, int table_n, const float* table,
+                                                         FarrowCoef* out, double* err) {
+    __shared__ double node_c[NH][NP][TAPS], node_q[NH][NQ][TAPS], cos_c[NP * NP], cos_q[NQ * NQ];
     __shared__ double emax[2][128];
     const int t = threadIdx.x;
-    if (t < NH * NP) {
-        const int h = t / NP, j = t % NP;
-        const double x = cos(M_PI * (j + 0.5) / NP);
-        interp_weights(kind, beta, table_n, table, 0.5 * (h + 0.5 + 0.5 * x), node_c[h][j]);
-    } else if (t < NH * NP + NH * NQ) {
-        const int h = (t - NH * NP) / NQ, j = (t - NH * NP) % NQ;
-        const double x = cos(M_PI * (j + 0.5) / NQ);
-        interp_weights(kind, beta, table_n, table, 0.5 * (h + 0.5 + 0.5 * x), node_q[h][j]);
+    constexpr int NODES = NH * (NP + NQ);
+    static_assert(NODES * TAPS <= 128 && NP * NP <= 16 && NQ * NQ <= 16, "a thread per (node, tap)");
+    if (t < NODES * TAPS) {
+        const int node = t / TAPS, m = t % TAPS;
+        const bool cub = node < NH * NP;
+        const int k = cub ? node : node - NH * NP, N = cub ? NP : NQ, h = k / N, j = k % N;
+        const double f = 0.5 * (h + 0.5 + 0.5 * cos(M_PI * (j + 0.5) / N));
+        (cub ? node_c[h][j] : node_q[h][j])[m] = interp_weight(kind, beta, table_n, table, f, m);
+    } else {
+        // T_k at the nodes: 128 - 112 threads for 16 + 9 cosines
+        for (int e = t - NODES * TAPS; e < NP * NP + NQ * NQ; e += 128 - NODES * TAPS) {
+            if (e < NP * NP)
+                cos_c[e] = cos(M_PI * (e / NP) * (e % NP + 0.5) / NP);
+            else
+                cos_q[e - NP * NP] = cos(M_PI * ((e - NP * NP) / NQ) * ((e - NP * NP) % NQ + 0.5) / NQ);
+        }
+    }
+    __syncthreads();
+    if (t < NODES && kind == SAS_INTERP_KAISER_SINC) {
+        double* w = t < NH * NP ? node_c[t / NP][t % NP] : node_q[(t - NH * NP) / NQ][(t - NH * NP) % NQ];
+        normalise_weights(w);
     }
     __syncthreads();
     if (t < NH * TAPS) {
         const int h = t / TAPS, m = t % TAPS;
         double mono[NP];
-        fit_half_tap<NP>(node_c[h], m, mono);
+        fit_half_tap<NP>(node_c[h], m, cos_c, mono);
         for (int p = 0; p < NP; ++p) out->c[h][m][p] = (float)mono[p];
     } else if (t < 2 * NH * TAPS) {
         const int h = (t - NH * TAPS) / TAPS, m = (t - NH * TAPS) % TAPS;
         double mono[NQ];
-        fit_half_tap<NQ>(node_q[h], m, mono);
+        fit_half_tap<NQ>(node_q[h], m, cos_q, mono);
         for (int p = 0; p < NQ; ++p) out->q[h][m][p] = (float)mono[p];
     }
+    if (!err) return;
     __syncthreads();
     // deviation of the (float-rounded) polynomials from the definition
     emax[0][t] = form_error<NP>(kind, beta, table_n, table, out->c);
@@ -315,7 +335,7 @@ __global__ void fit_interp_kernel(int kind, double beta, int table_n, const floa
     if (t < 2) {
         double m = 0.0;
         for (int k = 0; k < blockDim.x; ++k) m = fmax(m, emax[t][k]);
-        if (err) err[t] = m;
+        err[t] = m;
     }
 }
 
@@ -418,7 +438,6 @@ extern "C" int sas_geometry_create(const sas_nav* nav, const sas_signal* sig, vo
     const size_t o_st = o;  o = align256(o + 16);
     const size_t o_cu = o;  o = align256(o + 4 * 8);
     const size_t o_cf = o;  o = align256(o + sizeof(FarrowCoef));
-    const size_t o_fe = o;  o = align256(o + 2 * 8);
     cudaError_t e = cudaMalloc(&h->slab, o);
     if (e != cudaSuccess) {
         delete h;
@@ -438,7 +457,6 @@ extern "C" int sas_geometry_create(const sas_nav* nav, const sas_signal* sig, vo
     h->d_status = (uint32_t*)(b + o_st);
     h->d_cull = (unsigned long long*)(b + o_cu);
     h->d_coef = (FarrowCoef*)(b + o_cf);
-    h->d_fit_err = (double*)(b + o_fe);
     int rc = SAS_OK;
     auto ck = [&](cudaError_t err, const char* w) {
         if (rc == SAS_OK && err != cudaSuccess) rc = cuda_fail(err, w);
@@ -649,7 +667,7 @@ static int handle_fit(sas_geometry_t h, const sas_interp* it, cudaStream_t st) {
         h->fit_beta == it->kaiser_beta)
         return SAS_OK;
     h->fit_valid = 0;
-    int rc = fit_interp(it, h->d_coef, h->d_fit_err, st);
+    int rc = fit_interp(it, h->d_coef, nullptr, st);
     if (rc == SAS_OK && it->kind == SAS_INTERP_KAISER_SINC) {
         h->fit_valid = 1;
         h->fit_taps = it->taps;

@@ -264,7 +264,6 @@ struct sas_geometry_s {
     uint32_t* d_status;
     unsigned long long* d_cull;   // [4] ray-culling counts (candidate, computed, beam edge, -)
     sas::FarrowCoef* d_coef;
-    double* d_fit_err;
     int fit_valid;       // d_coef holds the Kaiser fit for (fit_taps, fit_beta)
     int fit_taps;
     double fit_beta;
