@@ -365,7 +365,8 @@ bool whiten_reg_dispatch(int n, bool apply, const float2* in, float2* out, long 
 constexpr int TVG_COLS = 8;
 constexpr int TVG_THREADS = 256;
 constexpr int TVG_RPI = TVG_THREADS / TVG_COLS;   // rows an iteration reads
-constexpr size_t TVG_SMEM = sizeof(unsigned) * TVG_COLS * 2048;
+constexpr int TVG_NH = TVG_COLS * 2048;    // counters: 2048 bins a column, or 2 x 1024
+constexpr size_t TVG_SMEM = sizeof(unsigned) * TVG_NH;
 
 __device__ __forceinline__ unsigned tvg_bits(float2 v) {
     return min(__float_as_uint(power_f32(v)), 0x7fffffffu);   // a NaN with the sign bit: the largest NaN
@@ -385,7 +386,7 @@ __device__ __forceinline__ void tvg_level(const float2* __restrict__ e, long lon
         p0 = prefix[2 * c] >> PSH;
         p1 = prefix[2 * c + 1] >> PSH;
     }
-    unsigned* h0 = h + (LEVEL == 1 ? c * NB : (2 * c) * NB);
+    unsigned* h0 = h + (LEVEL == 1 ? c : 2 * c) * NB;
     unsigned* h1 = h0 + NB;
     auto add = [&](unsigned bits) {
         const unsigned k = (bits >> BSH) & (NB - 1);
@@ -409,43 +410,61 @@ __device__ __forceinline__ void tvg_level(const float2* __restrict__ e, long lon
     for (; r < rows; r += TVG_RPI) add(tvg_bits(e[r * rstep * n + col]));
 }
 
+// The bin of the histogram h of NB bins that holds rank rk, and the count before it,
+// by one warp: the sums of runs of 32 bins (a conflict-free load and a warp sum each),
+// then the bins of the run that holds the rank.  (With a run of bins a lane, all lanes
+// hit one bank and a pick took 2 us; it came to a third of the TVG's time.)
+template <int NB>
+__device__ __forceinline__ void warp_pick(const unsigned* h, unsigned rk, unsigned& bin, unsigned& before) {
+    constexpr int HALVES = NB / 1024;          // 32 runs each
+    const int lane = threadIdx.x & 31;
+    auto scan = [&](unsigned v) {              // inclusive
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const unsigned y = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += y;
+        }
+        return v;
+    };
+    int run = 0;
+    unsigned below = 0u, base = 0u;
+#pragma unroll
+    for (int p = 0; p < HALVES; ++p) {
+        unsigned mine = 0u;                    // total of run 32 p + lane
+#pragma unroll 8
+        for (int r = 0; r < 32; ++r) {
+            const unsigned t = __reduce_add_sync(0xffffffffu, h[(32 * p + r) * 32 + lane]);
+            if (r == lane) mine = t;
+        }
+        const unsigned end = base + scan(mine);
+        const unsigned who = __ballot_sync(0xffffffffu, rk < end && rk >= end - mine);
+        if (who) {
+            const int l = __ffs(who) - 1;
+            run = 32 * p + l;
+            below = __shfl_sync(0xffffffffu, end - mine, l);
+        }
+        base = __shfl_sync(0xffffffffu, end, 31);
+    }
+    const unsigned c = h[run * 32 + lane], end = below + scan(c);
+    const unsigned hit = __ballot_sync(0xffffffffu, rk < end && rk >= end - c);
+    const int at = hit ? __ffs(hit) - 1 : 0;
+    bin = (unsigned)(run * 32 + at);
+    before = __shfl_sync(0xffffffffu, end - c, at);
+}
+
 // The bins of every (column, rank) holding the rank's residual: one warp per
-// (column, rank) pair, the lanes summing 32-bin slices and scanning.
+// (column, rank) pair.
 template <int LEVEL>
 __device__ __forceinline__ void tvg_pick(const unsigned* h, unsigned* prefix, unsigned* rank) {
-    constexpr int NB = LEVEL == 1 ? 2048 : 1024, PER = NB / 32, SH = LEVEL == 1 ? 20 : (LEVEL == 2 ? 10 : 0);
+    constexpr int NB = LEVEL == 1 ? 2048 : 1024, SH = LEVEL == 1 ? 20 : (LEVEL == 2 ? 10 : 0);
     const int lane = threadIdx.x & 31;
     for (int pr = threadIdx.x >> 5; pr < 2 * TVG_COLS; pr += TVG_THREADS / 32) {
         const int c = pr >> 1;
-        const unsigned* hh = h + (LEVEL == 1 ? c * NB : pr * NB);   // level 1: one histogram a column
-        const unsigned rk = rank[pr];
-        unsigned tot = 0u;
-        for (int k = 0; k < PER; ++k) tot += hh[lane * PER + k];
-        unsigned x = tot;
-        for (int o = 1; o < 32; o <<= 1) {
-            const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        unsigned below = x - tot;
-        const bool mine = rk >= below && rk - below < tot;
-        unsigned bin = 0u, before = 0u;
-        if (mine) {
-            for (int k = 0; k < PER; ++k) {
-                const unsigned hk = hh[lane * PER + k];
-                if (rk - below < hk) {
-                    bin = lane * PER + k;
-                    before = below;
-                    break;
-                }
-                below += hk;
-            }
-        }
-        const unsigned who = __ballot_sync(0xffffffffu, mine);
-        const int src = who ? __ffs(who) - 1 : 0;
-        bin = __shfl_sync(0xffffffffu, bin, src);
-        before = __shfl_sync(0xffffffffu, before, src);
+        unsigned bin, before;
+        // level 1: one histogram a column
+        warp_pick<NB>(h + (LEVEL == 1 ? c : pr) * NB, rank[pr], bin, before);
         if (lane == 0) {
-            rank[pr] = rk - before;
+            rank[pr] -= before;
             prefix[pr] |= bin << SH;
         }
     }
@@ -459,7 +478,7 @@ __global__ void __launch_bounds__(TVG_THREADS, 2) tvg_select_kernel(const float2
                                                                    long long rstep, int n, unsigned r_lo,
                                                                    unsigned r_hi, double* __restrict__ med,
                                                                    uint2* __restrict__ bracket) {
-    extern __shared__ unsigned tvg_h[];                       // TVG_COLS x 2048 counters
+    extern __shared__ unsigned tvg_h[];                       // TVG_NH counters
     __shared__ unsigned prefix[2 * TVG_COLS], rank[2 * TVG_COLS];   // index 2 c + r
     const int col = blockIdx.x * TVG_COLS + (int)(threadIdx.x % TVG_COLS);
     const bool colok = col < n;
@@ -467,19 +486,19 @@ __global__ void __launch_bounds__(TVG_THREADS, 2) tvg_select_kernel(const float2
         prefix[threadIdx.x] = 0u;
         rank[threadIdx.x] = (threadIdx.x & 1) ? r_hi : r_lo;
     }
-    for (int t = threadIdx.x; t < TVG_COLS * 2048; t += TVG_THREADS) tvg_h[t] = 0u;
+    for (int t = threadIdx.x; t < TVG_NH; t += TVG_THREADS) tvg_h[t] = 0u;
     __syncthreads();
     tvg_level<1>(e, rows, rstep, n, col, colok, tvg_h, prefix);
     __syncthreads();
     tvg_pick<1>(tvg_h, prefix, rank);
     __syncthreads();
-    for (int t = threadIdx.x; t < TVG_COLS * 2048; t += TVG_THREADS) tvg_h[t] = 0u;
+    for (int t = threadIdx.x; t < TVG_NH; t += TVG_THREADS) tvg_h[t] = 0u;
     __syncthreads();
     tvg_level<2>(e, rows, rstep, n, col, colok, tvg_h, prefix);
     __syncthreads();
     tvg_pick<2>(tvg_h, prefix, rank);
     __syncthreads();
-    for (int t = threadIdx.x; t < TVG_COLS * 2048; t += TVG_THREADS) tvg_h[t] = 0u;
+    for (int t = threadIdx.x; t < TVG_NH; t += TVG_THREADS) tvg_h[t] = 0u;
     __syncthreads();
     tvg_level<3>(e, rows, rstep, n, col, colok, tvg_h, prefix);
     __syncthreads();
@@ -550,40 +569,18 @@ __global__ void __launch_bounds__(TVG_THREADS) tvg_collect_kernel(const float2* 
 
 // One radix level's pick for a block selecting two ranks of one column: warp
 // r (r = 0, 1) finds the bin of h holding rank r's residual (level 0: one
-// histogram of NB bins for both; later levels: 1024 bins per rank at h + 1024 r),
-// appends it to pre[r] at bit SH and keeps the rank within the bin.
-__device__ void tvg_block_pick(const unsigned* h, int L, int NB, int SH, unsigned* pre, unsigned* rk) {
+// histogram of 2048 bins for both; later levels: 1024 bins per rank), appends it
+// to pre[r] at bit SH and keeps the rank within the bin.
+__device__ void tvg_block_pick(const unsigned* h, int L, int SH, unsigned* pre, unsigned* rk) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     if (wid >= 2) return;
-    const unsigned* hh = h + (L == 0 ? 0 : wid * 1024);
-    const int PER = NB / 32;
-    const unsigned want = rk[wid];
-    unsigned tot = 0u;
-    for (int k = 0; k < PER; ++k) tot += hh[lane * PER + k];
-    unsigned x = tot;
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    unsigned bl = x - tot, bin = 0u, before = 0u;
-    const bool mine = want >= bl && want - bl < tot;
-    if (mine) {
-        for (int k = 0; k < PER; ++k) {
-            const unsigned hk = hh[lane * PER + k];
-            if (want - bl < hk) {
-                bin = lane * PER + k;
-                before = bl;
-                break;
-            }
-            bl += hk;
-        }
-    }
-    const unsigned who = __ballot_sync(0xffffffffu, mine);
-    const int src = who ? __ffs(who) - 1 : 0;
-    bin = __shfl_sync(0xffffffffu, bin, src);
-    before = __shfl_sync(0xffffffffu, before, src);
+    unsigned bin, before;
+    if (L == 0)
+        warp_pick<2048>(h, rk[wid], bin, before);
+    else
+        warp_pick<1024>(h + wid * 1024, rk[wid], bin, before);
     if (lane == 0) {
-        rk[wid] = want - before;
+        rk[wid] -= before;
         pre[wid] |= bin << SH;
     }
 }
@@ -621,7 +618,7 @@ __global__ void __launch_bounds__(256) tvg_bracket_select_kernel(const unsigned*
             if (L > 0 && (b >> PSH) == p1) atomicAdd(&h[1024 + k], 1u);
         }
         __syncthreads();
-        tvg_block_pick(h, L, NB, SH, pre, rk);
+        tvg_block_pick(h, L, SH, pre, rk);
         __syncthreads();
     }
     if (threadIdx.x == 0) med[col] = 0.5 * ((double)__uint_as_float(pre[0]) + (double)__uint_as_float(pre[1]));
@@ -662,7 +659,7 @@ __global__ void __launch_bounds__(256) tvg_column_select_kernel(const float2* __
         }
         for (; r < rows; r += 256) add(tvg_bits(e[r * n + col]));
         __syncthreads();
-        tvg_block_pick(h, L, NB, SH, pre, rk);
+        tvg_block_pick(h, L, SH, pre, rk);
         __syncthreads();
     }
     if (threadIdx.x == 0) med[col] = 0.5 * ((double)__uint_as_float(pre[0]) + (double)__uint_as_float(pre[1]));
@@ -951,8 +948,24 @@ extern "C" int sas_matched_filter(const void* d_raw, int64_t rows, int32_t n, co
     }
     if (rows == 0) return SAS_OK;
     cudaStream_t st = (cudaStream_t)stream;
-    int NF = 256;
-    while (NF < 4 * L && NF < fftdev::MAX_N) NF *= 2;        // at least 3/4 of each block is output
+    // block length: the least time for ceil(n / M) blocks of NF points, M = NF - L + 1
+    // outputs each, from the measured time a point (8192 rows of 16384 samples: 256
+    // points 26.7 ps, then 38, 40, 39, 44, 60 and 68; one exchange at 256, two to 4096,
+    // three beyond).  L = 200: 2048 points (714 us; 1024, the shortest with 3/4 of a block
+    // output: 840 us)
+    static const double point_cost[7] = {0.69, 0.97, 1.03, 1.0, 1.13, 1.55, 1.75};
+    int NF = fftdev::MAX_N;
+    double best = 0.0;
+    for (int k = 6; k >= 0; --k) {
+        const int nf = 256 << k;
+        if (nf < 2 * L && k < 6) break;
+        const int m = nf - L + 1;
+        const double cost = (double)((n + m - 1) / m) * nf * point_cost[k];
+        if (k == 6 || cost <= best) {
+            best = cost;
+            NF = nf;
+        }
+    }
     const int M = NF - L + 1;
     const int nblk = (int)((n + M - 1) / M);
     float2* Pc = nullptr;
