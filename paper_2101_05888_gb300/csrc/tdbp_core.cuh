@@ -352,7 +352,36 @@ __device__ __forceinline__ PairGeoDF pair_geo_df(const KParams& p, const dfl* X0
     }
     return G;
 }
-__device__ __forceinline__ int pair_record_df(const KParams& p, const PairGeoDF& G, float* rc, int stride) {
+// v != nullptr: the receiver's velocity during reception (Sec. II-D).  With beta = v / c
+// the two-way path s = c tau of the tile centre solves (s - |R_T|)^2 = |R_R - beta s|^2,
+//   s = (|R_T| - rho + sqrt((|R_T| - rho)^2 - (1 - beta^2)(|R_T|^2 - |R_R|^2))) / (1 - beta^2),
+// rho = R_R . beta, and R_R is then taken from the receiver's position at that time (an FP64
+// fixed point in its place kept the producer warp on the slow FP64 pipe: the stripmap
+// with motion ran at 0.76 of its rate without).
+__device__ __forceinline__ int pair_record_df(const KParams& p, PairGeoDF G, float* rc, int stride,
+                                              const double* v = nullptr) {
+    if (v) {
+        dfl b[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const float2 s = df_split(v[k] * p.inv_c);
+            b[k] = dfl{s.x, s.y};
+            rc[(F_BRX + k) * stride] = 2.0f * df_float(G.R[k]);
+            rc[(F_VX + k) * stride] = df_float(b[k]);
+        }
+        auto dot = [](const dfl* x, const dfl* y) {
+            return df_add(df_add(df_mul(x[0], y[0]), df_mul(x[1], y[1])), df_mul(x[2], y[2]));
+        };
+        const dfl one{1.0f, 0.0f}, b2 = dot(b, b), rho = dot(G.R, b), T2 = dot(G.T, G.T), R2 = dot(G.R, G.R);
+        const dfl m = df_add(df_sqrt(T2), df_neg(rho));
+        const dfl disc = df_add(df_mul(m, m), df_neg(df_mul(df_add(one, df_neg(b2)), df_add(T2, df_neg(R2)))));
+        // 1 / (1 - beta^2) = 1 + beta^2 + beta^4 (beta^6 ~ 1e-18)
+        const dfl inv = df_add(one, df_add(b2, df_mul(b2, b2)));
+        const dfl s = df_mul(df_add(m, df_sqrt(disc)), inv);
+#pragma unroll
+        for (int k = 0; k < 3; ++k) G.R[k] = df_add(G.R[k], df_neg(df_mul(b[k], s)));
+        rc[F_RV * stride] = df_float(dot(G.R, b));
+    }
     const dfl nT2 = df_add(df_add(df_mul(G.T[0], G.T[0]), df_mul(G.T[1], G.T[1])), df_mul(G.T[2], G.T[2]));
     const dfl nR2 = df_add(df_add(df_mul(G.R[0], G.R[0]), df_mul(G.R[1], G.R[1])), df_mul(G.R[2], G.R[2]));
     const dfl nT = df_sqrt(nT2), nR = df_sqrt(nR2);
@@ -898,8 +927,8 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
         // before it expands stage k, group by group, into the Farrow buffers the
         // consumers read; a descriptor per buffer tells them which pairs it holds.
         const double X0 = p.x0 + cx * p.dx, Y0 = p.y0 + cy * p.dy, Z0 = Zc;
-        // double-float reference terms for the stop-and-hop straight-path model
-        constexpr bool DFREC = !MOTION && !REFRACT;
+        // double-float reference terms for straight paths
+        constexpr bool DFREC = !REFRACT;
         dfl X0d[3];
         {
             const float2 a = df_split(X0), b = df_split(Y0), c = df_split(Z0);
@@ -993,9 +1022,9 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
                                                Zc, rc, 1, LT0, LR0);
                     int base;
                     if constexpr (DFREC)
-                        base = pair_record_df(p, Gd, rc, 1);
+                        base = pair_record_df(p, Gd, rc, 1, MOTION ? p.vel + 3 * (size_t)iv : nullptr);
                     else
-                        base = pair_record(p, Gv, rc, 1, MOTION ? p.vel + 3 * (size_t)iv : nullptr, LT0, LR0);
+                        base = pair_record(p, Gv, rc, 1, nullptr, LT0, LR0);
                     const int seg_start = base - (((base % p.seg_align) + p.seg_align) % p.seg_align);
                     rc[F_OFF] = __int_as_float(base - seg_start);
                     rc[F_SCALE] = p.scale ? p.scale[qv] : 1.0f;
