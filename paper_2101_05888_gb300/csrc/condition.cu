@@ -525,8 +525,10 @@ __global__ void __launch_bounds__(TVG_THREADS, 2) tvg_select_kernel(const float2
 // all its rows by a block of its own (the three radix levels), so the result
 // is exact in every case.
 constexpr int TVG_CAP = 8192;
-constexpr long long TVG_BRACKET_MIN_ROWS = 16384;   // fewer rows: the three-level select directly
-constexpr long long TVG_SAMPLE = 2048;              // rows of the sample (about)
+constexpr long long TVG_BRACKET_MIN_ROWS = 8192;    // fewer rows: the three-level select directly (5000 x 2048: as fast)
+// rows of the sample (about): the bracket holds 4 sqrt(sample) / sample of the rows,
+// which has to stay well below TVG_CAP
+constexpr long long TVG_SAMPLE = 2048, TVG_SAMPLE_FEW = 1024, TVG_FEW_ROWS = 32768;
 
 __global__ void __launch_bounds__(TVG_THREADS) tvg_collect_kernel(const float2* __restrict__ e, long long rows, int n,
                                                                   const uint2* __restrict__ bracket,
@@ -1080,7 +1082,7 @@ extern "C" int sas_tvg(const void* d_in, void* d_out, int64_t rows, int32_t n, d
                                                                  (unsigned)(rows / 2), med, nullptr);
     } else {
         // the sample: every rstep-th row (m of them), its ranks m/2 -+ about four standard deviations
-        const long long rstep = rows / TVG_SAMPLE, m = (rows + rstep - 1) / rstep;
+        const long long rstep = rows / (rows < TVG_FEW_ROWS ? TVG_SAMPLE_FEW : TVG_SAMPLE), m = (rows + rstep - 1) / rstep;
         const long long d = (long long)std::ceil(2.0 * std::sqrt((double)m)) + 1;
         const unsigned k_lo = (unsigned)std::max(0LL, (m - 1) / 2 - d), k_hi = (unsigned)std::min(m - 1, m / 2 + d);
         // scratch: brackets, candidates, counts, flags
