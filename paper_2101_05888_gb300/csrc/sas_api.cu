@@ -82,24 +82,32 @@ int encode_echo_map(CUtensorMap* map, const void* base, int elem_bytes, int Ns, 
 // ---------------------------------------------------------------------------
 // Sensor positions (Sec. II-C): x_TX,i = p_i + dp_i + R_i l_TX, x_RX,i,c = p_i + dp_i + R_i l_c,
 // with R_i the attitude rotation of Eq. 2 (attitude_rotation).
-__global__ void geometry_kernel(int P, int C, const double* __restrict__ pos, const double* __restrict__ att,
+// One warp a ping: three lanes take the angles' sines and cosines, then a lane a
+// sensor (a thread a ping took 24 us for 256 pings x 16 receivers, one long chain of FP64
+// operations; autofocus moves the sensors twice a step).
+constexpr int GEO_WARPS = 4;
+__global__ void __launch_bounds__(32 * GEO_WARPS) geometry_kernel(int P, int C, const double* __restrict__ pos, const double* __restrict__ att,
                                 const double* __restrict__ lever, const double* __restrict__ off,
                                 double* __restrict__ tx, double* __restrict__ rx, float* __restrict__ rotc,
                                 float2* __restrict__ txs, float2* __restrict__ rxs) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= P) return;
-    double R[9];
-    attitude_rotation(att[3 * i + 0], att[3 * i + 1], att[3 * i + 2], R);
+    const int i = blockIdx.x * GEO_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (i >= P) return;   // whole warps
+    double R[9], sn, cs;
+    sincos(att[3 * i + lane % 3], &sn, &cs);
+    rotation_of(__shfl_sync(0xffffffffu, sn, 0), __shfl_sync(0xffffffffu, cs, 0), __shfl_sync(0xffffffffu, sn, 1),
+                __shfl_sync(0xffffffffu, cs, 1), __shfl_sync(0xffffffffu, sn, 2), __shfl_sync(0xffffffffu, cs, 2), R);
     const double b0 = pos[3 * i] + off[3 * i], b1 = pos[3 * i + 1] + off[3 * i + 1],
                  b2 = pos[3 * i + 2] + off[3 * i + 2];
     // columns 0 and 1 of R: body-frame components (R^T v).x, (R^T v).y of a NED vector v
-    rotc[6 * i + 0] = (float)R[0];
-    rotc[6 * i + 1] = (float)R[3];
-    rotc[6 * i + 2] = (float)R[6];
-    rotc[6 * i + 3] = (float)R[1];
-    rotc[6 * i + 4] = (float)R[4];
-    rotc[6 * i + 5] = (float)R[7];
-    for (int c = -1; c < C; ++c) {
+    if (lane == 0) {
+        rotc[6 * i + 0] = (float)R[0];
+        rotc[6 * i + 1] = (float)R[3];
+        rotc[6 * i + 2] = (float)R[6];
+        rotc[6 * i + 3] = (float)R[1];
+        rotc[6 * i + 4] = (float)R[4];
+        rotc[6 * i + 5] = (float)R[7];
+    }
+    for (int c = lane - 1; c < C; c += 32) {
         const double* l = lever + 3 * (c + 1);
         double* o = (c < 0) ? tx + 3 * (size_t)i : rx + 3 * ((size_t)i * C + c);
         o[0] = b0 + R[0] * l[0] + R[1] * l[1] + R[2] * l[2];
@@ -111,7 +119,7 @@ __global__ void geometry_kernel(int P, int C, const double* __restrict__ pos, co
 }
 
 static int run_geometry(sas_geometry_t h, cudaStream_t st) {
-    geometry_kernel<<<(h->P + 127) / 128, 128, 0, st>>>(h->P, h->C, h->d_pos, h->d_att, h->d_lever, h->d_off,
+    geometry_kernel<<<(h->P + GEO_WARPS - 1) / GEO_WARPS, 32 * GEO_WARPS, 0, st>>>(h->P, h->C, h->d_pos, h->d_att, h->d_lever, h->d_off,
                                                         h->d_tx, h->d_rx, h->d_rotc, h->d_txs, h->d_rxs);
     SAS_CUDA(cudaGetLastError());
     return SAS_OK;

@@ -53,14 +53,18 @@ __device__ __forceinline__ unsigned row_index(unsigned raw, unsigned last, uint3
 //   [ ct cps,  cps st sph - cph sps,  cph cps st + sph sps ]
 //   [ ct sps,  cph cps + st sph sps,  cph st sps - cps sph ]
 //   [ -st,     ct sph,                ct cph               ]
+__device__ __forceinline__ void rotation_of(double sph, double cph, double sth, double cth, double sps, double cps,
+                                            double R[9]) {
+    R[0] = cth * cps; R[1] = cps * sth * sph - cph * sps; R[2] = cph * cps * sth + sph * sps;
+    R[3] = cth * sps; R[4] = cph * cps + sth * sph * sps; R[5] = cph * sth * sps - cps * sph;
+    R[6] = -sth;      R[7] = cth * sph;                   R[8] = cth * cph;
+}
 __device__ __forceinline__ void attitude_rotation(double roll, double pitch, double yaw, double R[9]) {
     double sph, cph, sth, cth, sps, cps;
     sincos(roll, &sph, &cph);
     sincos(pitch, &sth, &cth);
     sincos(yaw, &sps, &cps);
-    R[0] = cth * cps; R[1] = cps * sth * sph - cph * sps; R[2] = cph * cps * sth + sph * sps;
-    R[3] = cth * sps; R[4] = cph * cps + sth * sph * sps; R[5] = cph * sth * sps - cps * sph;
-    R[6] = -sth;      R[7] = cth * sph;                   R[8] = cth * cph;
+    rotation_of(sph, cph, sth, cth, sps, cps, R);
 }
 
 constexpr int TAPS = 8;

@@ -824,7 +824,7 @@ inline size_t smem_bytes(int slot_bytes, int npos_pad, int nrec, int row_bytes, 
            + (size_t)nbuf * GROUP * npos_pad * NH * row_bytes  // Farrow rows
            + (size_t)NRS * PAIRS * nrec * 4                    // records
            + (size_t)NH * TAPS * NP * 4                        // coefficients
-           + (size_t)NCW * 4 * 8                        // cross-warp reduction (gradient)
+           + (size_t)2 * NCW * 4 * 8                    // cross-warp reduction (gradient), two sets
            + (size_t)NBUF * 16                          // group descriptors
            + (size_t)(NSEG + NRS + 2 * NBUF) * 8 + 16;  // mbarriers, abort flag
 }
@@ -867,9 +867,9 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
     float* rec = reinterpret_cast<float*>(ebuf + (size_t)nbuf * GROUP * ebuf_pair);   // [NRS][PAIRS][KREC]
     float* coef_s = rec + NRS * PAIRS * KREC;                            // [NH][TAPS][NP]
     // every part so far has a size that is a multiple of 16 bytes (see smem_bytes)
-    double* wred = reinterpret_cast<double*>(coef_s + NH * TAPS * NP);    // [NCW][4]
+    double* wred = reinterpret_cast<double*>(coef_s + NH * TAPS * NP);    // [2][NCW][4]
     // [NBUF] group descriptors (written before, read after the efull barrier)
-    int4* gdesc = reinterpret_cast<int4*>(wred + NCW * 4);
+    int4* gdesc = reinterpret_cast<int4*>(wred + 2 * NCW * 4);
     uint64_t* full = reinterpret_cast<uint64_t*>(gdesc + NBUF);          // [NSEG] copies landed + records
     uint64_t* rempty = full + NSEG;                                      // [NRS] consumers done with records
     uint64_t* efull = rempty + NRS;                                      // [NBUF] Farrow rows written
@@ -1257,6 +1257,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
     // gradient with seabed refraction: the current ping's transmitter-leg blocks
     float4 ftr0 = make_float4(0.f, 0.f, 0.f, 0.f), ftr1 = ftr0, ftr2 = ftr0;
     bool ftrefr = false;
+    int nflush = 0;
     auto flush_ping = [&](int ping) {
         if (MODE != MODE_OFFSET_GRAD) return;
         const float tTv = DIM3 ? tT2 : tT1;
@@ -1296,27 +1297,26 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
             rsum[MODE == MODE_OFFSET_GRAD ? s : 0] = 0.f;
         }
         (void)hy;
-        double v0 = gacc0, v1 = gacc1, v2 = gacc2;
+        // warp sums of the three components by recursive halving (FP64 is slow here: 6
+        // additions a lane instead of 15); lanes 0, 8 and 16 end with x, y and z
+        const double v0 = gacc0, v1 = gacc1, v2 = gacc2;
         gacc0 = gacc1 = gacc2 = 0.f;
+        const bool up = lane & 16, mid = lane & 8;
+        const double a = (up ? v2 : v0) + __shfl_xor_sync(0xffffffffu, up ? v0 : v2, 16);
+        const double b = (up ? 0.0 : v1) + __shfl_xor_sync(0xffffffffu, up ? v1 : 0.0, 16);
+        double r = (mid ? b : a) + __shfl_xor_sync(0xffffffffu, mid ? a : b, 8);
 #pragma unroll
-        for (int o = 16; o; o >>= 1) {
-            v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-            v1 += __shfl_xor_sync(0xffffffffu, v1, o);
-            v2 += __shfl_xor_sync(0xffffffffu, v2, o);
-        }
-        const int cw = ct >> 5;
-        if (lane == 0) {
-            wred[cw * 4 + 0] = v0;
-            wred[cw * 4 + 1] = v1;
-            wred[cw * 4 + 2] = v2;
-        }
+        for (int o = 4; o; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+        // two sets of warp sums in turn: the barrier of the next ping stands between the
+        // reads of this set and its next writes
+        double* wr = wred + (nflush++ & 1) * NCW * 4;
+        if ((lane & 7) == 0) wr[(ct >> 5) * 4 + (lane >> 3)] = r;
         named_bar_sync(BAR_CONS, NCONS);
         if (ct < 3) {
             double sum = 0.0;
-            for (int w2 = 0; w2 < NCW; ++w2) sum += wred[w2 * 4 + ct];
+            for (int w2 = 0; w2 < NCW; ++w2) sum += wr[w2 * 4 + ct];
             p.partials[((size_t)tile * p.P + ping) * 3 + ct] = sum * (double)p.grad_scale;
         }
-        named_bar_sync(BAR_CONS, NCONS);
         (void)tNT;
     };
 
