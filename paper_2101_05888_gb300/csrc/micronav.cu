@@ -1164,12 +1164,19 @@ extern "C" int sas_dpc_solve(const sas_dpc_problem* pr, double* d_vy, double* d_
         else
             cost = hacc[0];
     }
-    double mu = 1e-3, last_step = 0.0;
-    int polish = 0;   // steps taken after the loss stalled
+    // The loss of a few 1e5 residuals of 1e-4 m, differences of 100 m paths, rounds at
+    // about 3e-12 of its value, so below LOSS_NOISE it cannot tell two points apart: near
+    // the minimum Newton's steps shrink a hundredfold each while the loss moves up or
+    // down at random (judged by it, half of them were repeated with growing damping, 20
+    // to 30 trials long).  Such a step is taken when it shrinks, and the search ends
+    // once steps stop shrinking.
+    constexpr double LOSS_NOISE = 1e-11;
+    double mu = 1e-3, last_step = INFINITY;
+    int flat = 0;   // trials within the noise that did not shrink
     for (int it = 0; rc == SAS_OK && it < max_iter; ++it) {
-        bool accepted = false, stalled = false;
-        double trial = cost, step = 0.0;
-        for (int tries = 0; tries < 40 && rc == SAS_OK; ++tries) {
+        bool accepted = false, done = false;
+        double trial = cost;
+        for (int tries = 0; tries < 40 && rc == SAS_OK && !done; ++tries) {
             // the step, and the normal equations at the trial point with its loss (needed
             // next when it is accepted, as it nearly always is): one read-back a trial
             cudaError_t e = cudaMemsetAsync(acc, 0, 4 * sizeof(double), st);
@@ -1184,31 +1191,26 @@ extern "C" int sas_dpc_solve(const sas_dpc_problem* pr, double* d_vy, double* d_
                 mu *= 10.0;
                 continue;
             }
-            step = hacc[2];
+            const double step = hacc[2];
             trial = hacc[0];
-            // a rise within the loss's rounding is no reason to reject a step: it would be
-            // repeated with more damping, tens of times
-            if (trial - cost <= (polish ? 1e-13 : 1e-14) * cost) {
+            const bool blind = std::fabs(trial - cost) <= LOSS_NOISE * cost, shrinks = step <= 0.5 * last_step;
+            if (blind && !shrinks) ++flat;
+            if (trial <= cost || (blind && shrinks)) {
                 std::swap(S.q, q_try);
                 std::swap(cur, nxt);
                 accepted = true;
-                stalled = (cost - trial) <= 1e-14 * cost || step == 0.0;
+                done = step == 0.0 || (blind && std::fabs(cost - trial) <= 1e-14 * cost && !shrinks) || flat >= 3;
+                last_step = step;
                 mu = std::max(mu / 3.0, 1e-15);
                 break;
             }
-            if (polish) break;
+            done = flat >= 3;
             mu *= 4.0;
         }
         if (rc != SAS_OK || !accepted) break;
         ++iters;
         cost = trial;
-        // once the loss cannot tell any more (its rounding hides 1e-7 of the weakly determined
-        // directions), up to three more steps while they keep shrinking
-        if (stalled || polish) {
-            if (step == 0.0 || polish == 3 || (polish && step > 0.5 * last_step)) break;
-            ++polish;
-            last_step = step;
-        }
+        if (done) break;
     }
     if (rc == SAS_OK) {
         dpc_velocities_kernel<<<blocks_for(pb.P, 128), 128, 0, st>>>(pb, S.q, d_vy, d_vz);
