@@ -192,6 +192,7 @@ __global__ void whiten_reduce_kernel(const double* __restrict__ part, int nparts
     const int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= n) return;
     double s = 0.0;
+#pragma unroll 16   // loads in flight; the sum stays in order
     for (int b = 0; b < nparts; ++b) s += part[(size_t)b * n + f];
     P[f] = s / (double)rows;
 }
@@ -201,6 +202,7 @@ __global__ void __launch_bounds__(1024) whiten_stats_kernel(const double* __rest
                                                             double* __restrict__ stats) {
     __shared__ double red[32], mn[32];
     double s = 0.0, pmin = 1.0 / 0.0;
+#pragma unroll 8
     for (int f = threadIdx.x; f < n; f += blockDim.x) {
         s += P[f];
         pmin = fmin(pmin, P[f]);
@@ -674,6 +676,7 @@ __global__ void __launch_bounds__(256) tvg_gain_kernel(const double* __restrict_
                                                        float* __restrict__ gain) {
     __shared__ double red[256];
     double s = 0.0;
+#pragma unroll 16   // loads in flight; the sum stays in order
     for (int t = threadIdx.x; t < n; t += blockDim.x) s += med[t];
     red[threadIdx.x] = s;
     __syncthreads();
