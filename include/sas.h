@@ -203,6 +203,9 @@ int sas_echo_download(sas_geometry_t h, void* d_out, void* cuda_stream);
 /* 2D backprojection onto the grid plane z = z0 (grid->nz must be 1).
  * d_image: complex64 [ny][nx], device.  accumulate = 0 overwrites the image,
  * 1 adds to it (e.g. to stream pings through several echo uploads).
+ * Small and middling grids are computed in several parts that are added in a fixed
+ * order (the image does not depend on the run); the parts take up to 70 MB of scratch
+ * that stays with the handle (stream-ordered memory while the stream is captured).
  * Errors: SAS_ERR_ARG, SAS_ERR_STATE (no echo), SAS_ERR_UNSUPPORTED (taps != 8,
  * a tile's delay span too long for the staging buffers), SAS_ERR_CUDA. */
 int sas_backproject_2d(sas_geometry_t h, const sas_grid* grid, const sas_interp* interp,

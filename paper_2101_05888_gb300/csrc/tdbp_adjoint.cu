@@ -3,7 +3,8 @@
 //    forward sum:  e_adj[i][c][floor u + k] += w_k(frac u) exp(-j 2 pi fc tau) I(x);
 //  * dispatch of the offset gradient (tdbp_vjp.cu).
 //
-// Linear adjoint, one CTA per tile (warp 0 computes the FP64 reference terms
+// Linear adjoint over straight 2D legs: adjoint2d_kernel below.  In 3D, with a beam,
+// receiver motion or refraction, one CTA per tile (warp 0 computes the reference terms
 // of 32 pairs at a time, warps 1..7 own 8 pixels each).  With the Farrow form
 // w_k(f) = sum_p coef[h][k][p] g^p on the half h of the sample interval the
 // per-pixel work is a scatter of g^p v (v = I(x) exp(-j 2 pi fc tau)) into

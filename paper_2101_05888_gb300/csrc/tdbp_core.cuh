@@ -11,8 +11,8 @@
 // with G = dL/dI* and u_T, u_R unit vectors from the sensors to the pixel.
 //
 // One CTA per image tile; warp 0 is the producer, warps 1..7 the consumers.
-//  * producer, one lane per (ping, channel) pair, 32 pairs a stage: FP64
-//    reference terms at the tile centre x0 (R = x0 - sensor, |R|, tau_ref,
+//  * producer, one lane per (ping, channel) pair, 32 pairs a stage: double-float
+//    (refraction: FP64) reference terms at the tile centre x0 (R = x0 - sensor, |R|, tau_ref,
 //    floor(u_ref), fraction, carrier phase mod 1) written to shared memory,
 //    and a 2D bulk tensor copy of the echo segment the tile can reach into a
 //    ring of NSEG stages, completion on an mbarrier (transaction bytes).
@@ -24,19 +24,17 @@
 //      minus 1/2), so s = sum_p g^p E_p^h[floor u] with
 //      E_p^h[i] = sum_m coef[h][m][p] e[i + k_m], computed once per (pair,
 //      tile) for both halves of every sample position the tile can reach:
-//      one row per half-sample position.  Complex64 echoes: E_0..E_3 in FP32,
-//      a 32-byte row read by two 16-byte loads.  16-bit echoes (rows
-//      normalised to |e| <= 1, so |E_p| stays near 1): E_0..E_3 in FP16, a
-//      16-byte row, and the forward Horner in packed FP16, the row scale
-//      applied afterwards in FP32.
+//      one row per half-sample position, E_0..E_3 in FP32 in two planes of
+//      16 bytes.  16-bit echoes in the forward pass: quadratics, E_0..E_2.
 //  * consumers, 8 pixels a thread, group after group:
 //    - per pixel and pair, with the pair's reference terms read by uniform
 //      16-byte loads: differential range dr = (2 R.d + |d|^2) / (|R + d| + |R|), an
 //      exact identity evaluated in FP32 on small quantities (d = x - x0); 2u
-//      and the phase from the reference values plus dr-derived offsets;
-//      floor/fraction on the FP32 pipe; the row (two 16-byte shared loads,
-//      or one for FP16 rows); cubic Horner in g; SFU rsqrt, rcp, sin, cos (the
-//      carrier phase in radians, taken directly while it stays within 512 rad).
+//      and the phase from the reference values plus dr-derived offsets
+//      (16-bit echoes over straight legs: a series along the thread's column of
+//      pixels instead, see leg_series); floor/fraction on the FP32 pipe; the row
+//      (two shared loads); Horner in g; SFU sin, cos (the carrier phase in
+//      radians, taken directly while it stays within 512 rad) and, a pixel, rsqrt, rcp.
 //    - the pixels of a warp form an 8 x 4 block (4 x 2 per quarter-warp), so
 //      the rows one 16-byte load instruction reads span fewer than 8
 //      consecutive half-sample positions (quarter-warp phases) and fall in
@@ -83,7 +81,11 @@ enum { GD_STAGE_END = 1, GD_LAST = 2, GD_EXACT = 4 };
 enum {
     F_RX, F_RY, F_RZ, F_NR2, F_NR, F_UF, F_PH, F_SCALE, F_TX, F_TY, F_TZ, F_NT2, F_NT, F_PING, F_FLAGS, F_OFF,
     F_C0X, F_C0Y, F_C0Z, F_C1X, F_C1Y, F_C1Z, F_PAD0, F_PAD1, F_VX, F_VY, F_VZ, F_RV, F_BRX, F_BRY, F_BRZ, F_PAD2,
-    NREC
+    // nine 16-byte blocks: the lanes of the producer, a record each, then store to
+    // different banks (eight blocks put all 32 lanes on one, a tenth of a pair's
+    // wavefronts in the pipe that binds the kernel: 64 x 32 -> 4096^2 in complex64
+    // 42.2 -> 41.5 ms)
+    NREC = F_PAD2 + 5
 };
 // pair flags: the whole tile lies inside the transmitter / receiver beam;
 // the transmitter / receiver leg refracts into the sediment for some pixel
@@ -817,7 +819,7 @@ constexpr int NPOS_FIXED = 60;
 static_assert(NPOS_FIXED % RUN == 0, "whole expansion runs");
 
 // shared memory with which two CTAs fit an SM
-constexpr size_t SMEM_TWO_CTAS = 113 * 1024;
+constexpr size_t SMEM_TWO_CTAS = 112 * 1024;
 
 inline size_t smem_bytes(int slot_bytes, int npos_pad, int nrec, int row_bytes, int nbuf) {
     return (size_t)NSEG * PAIRS * slot_bytes                   // echo segments
@@ -850,8 +852,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
     // rotation's cross terms are resolved once, when the tile is written)
     constexpr bool ACC2 = MODE == MODE_FORWARD && !REFRACT;
     constexpr int KREC = REFRACT ? NREC_REFR : NREC;   // record fields
-    // FP16 Farrow rows for 16-bit echoes in the forward pass; otherwise rows
-    // of FP32 E0, E1 and BF16 E2, E3
+    // quadratic rows for 16-bit echoes in the forward pass, otherwise cubic ones
     constexpr bool E16 = (MODE == MODE_FORWARD) && (sizeof(ET) == 4);
     constexpr int ROWB = E16 ? ROW24 : ROW32;
     constexpr int NPK = E16 ? NQ : NP;                 // coefficients of a row (cubic or quadratic)
