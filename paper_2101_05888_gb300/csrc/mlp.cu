@@ -406,7 +406,9 @@ extern "C" int sas_mlp_loss_grad(const float* d_theta, const float* d_frac, cons
     }
     cudaStream_t st = (cudaStream_t)stream;
     const int nb = (int)((n + SPB - 1) / SPB);
-    float* part_grad = (float*)d_work;
+    // from the next 16-byte boundary on (the kernel stores float4; the size's spare 256
+    // bytes cover the shift, so the caller's pointer may have any alignment of a float)
+    float* part_grad = (float*)(((uintptr_t)d_work + 15) & ~(uintptr_t)15);
     float* part_loss = part_grad + (size_t)nb * NPAR;
     const size_t smem = block_smem();
     SAS_CUDA(cudaFuncSetAttribute(mlp_block_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
