@@ -71,19 +71,23 @@ int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long slots, Setu
     const int slot_bytes = (slot_samples * elem + 127) / 128 * 128;
     // quadratic rows for 16-bit echoes in the forward pass, else cubic rows
     const int row_bytes = (mode == MODE_FORWARD && elem == 4) ? ROW24 : ROW32;
-    // two Farrow buffers instead of three where that lets a second CTA onto the SM (2D
-    // complex64 pixels of 1.6 to 2.4 cm at 40 kHz: 120 -> 101 KB)
     const int nrec = refract ? (int)NREC_REFR : (int)NREC;
-    int nbuf = NBUF;
-    if (smem_bytes(slot_bytes, npos_pad, nrec, row_bytes, 3) > SMEM_TWO_CTAS &&
-        smem_bytes(slot_bytes, npos_pad, nrec, row_bytes, 2) <= SMEM_TWO_CTAS)
-        nbuf = 2;
-    const size_t smem = smem_bytes(slot_bytes, npos_pad, nrec, row_bytes, nbuf);
-    if (smem > SMEM_TWO_CTAS) slots /= 2;    // one CTA an SM
-    if (smem > 227 * 1024) {
-        set_error("shared memory need %zu exceeds the per-block limit", smem);
+    const size_t smem3 = smem_bytes(slot_bytes, npos_pad, nrec, row_bytes, 3),
+                 smem2 = smem_bytes(slot_bytes, npos_pad, nrec, row_bytes, 2);
+    // spans are taken up to the one whose three buffers fill the block with records of
+    // eight 16-byte blocks and one set of warp sums, whatever else has been added since
+    constexpr size_t LIMIT = 227 * 1024;
+    const size_t added = NCW * 4 * 8 + (refract ? 0 : (size_t)NRS * PAIRS * (NREC - 32) * 4);
+    if (smem3 > LIMIT + added) {
+        set_error("shared memory need %zu exceeds the per-block limit", smem3);
         return SAS_ERR_UNSUPPORTED;
     }
+    // two Farrow buffers instead of three where three do not fit (16-bit offset gradient,
+    // 2D pixels of 5.7 to 6.05 cm at 40 kHz), or where two let a second CTA onto the SM
+    // (2D complex64 pixels of 1.6 to 2.4 cm: 120 -> 101 KB)
+    const int nbuf = smem3 > LIMIT || (smem3 > SMEM_TWO_CTAS && smem2 <= SMEM_TWO_CTAS) ? 2 : NBUF;
+    const size_t smem = nbuf == 2 ? smem2 : smem3;
+    if (smem > SMEM_TWO_CTAS) slots /= 2;    // one CTA an SM
     KParams& prm = S.prm;
     prm = KParams{};
     prm.tx = h->d_tx;
