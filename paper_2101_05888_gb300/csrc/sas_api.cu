@@ -27,6 +27,34 @@ int cuda_fail(cudaError_t e, const char* what) {
     return e == cudaErrorMemoryAllocation ? SAS_ERR_OOM : SAS_ERR_CUDA;
 }
 
+cudaError_t call_scratch(HandleScratch& s, size_t bytes, cudaStream_t st, void** p, bool* own) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    *own = false;
+    cudaError_t e = cudaStreamIsCapturing(st, &cs);
+    if (e != cudaSuccess) return e;
+    if (cs != cudaStreamCaptureStatusNone) {
+        e = cudaMallocAsync(p, bytes, st);
+        *own = e == cudaSuccess;
+        return e;
+    }
+    if (s.bytes < bytes) {
+        if (s.p) {
+            e = cudaStreamSynchronize(st);
+            if (e != cudaSuccess) return e;
+            cudaFree(s.p);
+            s = HandleScratch{nullptr, 0};
+        }
+        e = cudaMalloc(&s.p, bytes);
+        if (e != cudaSuccess) {
+            s.p = nullptr;
+            return e;
+        }
+        s.bytes = bytes;
+    }
+    *p = s.p;
+    return cudaSuccess;
+}
+
 int sm_count() {
     static int cached[64] = {0};
     int dev = 0;
@@ -554,7 +582,8 @@ extern "C" int sas_geometry_destroy(sas_geometry_t h) {
     cudaDeviceSynchronize();
     if (h->d_echo) cudaFree(h->d_echo);
     if (h->d_scale) cudaFree(h->d_scale);
-    if (h->d_scratch) cudaFree(h->d_scratch);
+    if (h->partials.p) cudaFree(h->partials.p);
+    if (h->planes.p) cudaFree(h->planes.p);
     if (h->slab) cudaFree(h->slab);
     delete h;
     return SAS_OK;

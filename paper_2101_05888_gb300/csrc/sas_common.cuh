@@ -243,6 +243,13 @@ constexpr float FLOOR_MAGIC = 12582912.0f;  // 1.5 * 2^23
 // ---------------------------------------------------------------------------
 // Handle
 
+namespace sas {
+struct HandleScratch {
+    void* p;
+    size_t bytes;
+};
+}  // namespace sas
+
 struct sas_geometry_s {
     int device;
     int P, C, Ns;
@@ -276,9 +283,9 @@ struct sas_geometry_s {
     float* d_scale;    // [P][C] (16-bit storage)
     int echo_dtype;    // -1 = none
     size_t echo_bytes;
-    // adjoint / VJP scratch (grown on demand)
-    void* d_scratch;
-    size_t scratch_bytes;
+    // scratch, grown on demand: the offset gradient's partial sums, the forward pass's
+    // planes (two buffers, so that neither call's growth replaces the other's)
+    sas::HandleScratch partials, planes;
     // failure-detection test hook
     int debug_skip_copies;
     int32_t debug_wait_ms;
@@ -310,5 +317,11 @@ int launch_adjoint(const AdjointArgs& a);
 int encode_echo_map(CUtensorMap* map, const void* base, int elem_bytes, int Ns, int rows, int box_len);
 
 int sm_count();
+
+// `bytes` of device memory for one call on `st`: the handle's buffer s, grown when it is
+// too small, or, while the stream is being captured, stream-ordered memory (*own: to be
+// freed on the stream after use) -- a graph must not keep a pointer that a later call of
+// the handle may replace.
+cudaError_t call_scratch(HandleScratch& s, size_t bytes, cudaStream_t st, void** p, bool* own);
 
 }  // namespace sas

@@ -253,35 +253,6 @@ __global__ void __launch_bounds__(256) sum_splits_kernel(const float2* __restric
 
 }  // namespace core
 
-// Planes for the parts of a split launch: the handle's scratch, or, while the
-// stream is being captured, stream-ordered memory (*own: to be freed after
-// use) -- a graph must not keep a pointer that a later call may replace.  nullptr:
-// no memory (the error is cleared).
-static float2* split_planes(sas_geometry_t h, size_t bytes, cudaStream_t st, bool* own) {
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    void* p = nullptr;
-    *own = false;
-    if (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
-        if (h->scratch_bytes >= bytes) return (float2*)h->d_scratch;
-        if (h->d_scratch) {
-            if (cudaStreamSynchronize(st) != cudaSuccess) return nullptr;
-            cudaFree(h->d_scratch);
-            h->d_scratch = nullptr;
-            h->scratch_bytes = 0;
-        }
-        if (cudaMalloc(&h->d_scratch, bytes) == cudaSuccess) {
-            h->scratch_bytes = bytes;
-            return (float2*)h->d_scratch;
-        }
-        h->d_scratch = nullptr;
-    } else if (cudaMallocAsync(&p, bytes, st) == cudaSuccess) {
-        *own = true;
-        return (float2*)p;
-    }
-    (void)cudaGetLastError();
-    return nullptr;
-}
-
 int launch_forward(const ForwardArgs& a) {
     core::Setup S;
     int rc = core::prepare(a.h, a.grid, a.dim3, 2LL * sm_count(), S);
@@ -294,8 +265,9 @@ int launch_forward(const ForwardArgs& a) {
     // and it had to be cleared first); at most 16 x slots tiles' worth of planes
     const size_t npix = (size_t)a.grid.nx * a.grid.ny * S.prm.nz;
     bool own = false;
-    float2* parts = split_planes(a.h, sizeof(float2) * npix * S.prm.nsplit, a.stream, &own);
-    if (!parts) {   // no memory for the planes: one CTA a tile
+    float2* parts = nullptr;
+    if (call_scratch(a.h->planes, sizeof(float2) * npix * S.prm.nsplit, a.stream, (void**)&parts, &own) != cudaSuccess) {
+        (void)cudaGetLastError();   // no memory for the planes: one CTA a tile
         rc = core::prepare(a.h, a.grid, a.dim3, 0, S);
         if (rc != SAS_OK) return rc;
         S.prm.image = a.image;

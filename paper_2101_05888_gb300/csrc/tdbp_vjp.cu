@@ -76,27 +76,24 @@ int launch_offset_grad(sas_geometry_t h, const sas_grid& g, const float2* grad_i
     if (rc != SAS_OK) return rc;
     const long long ntiles = (long long)S.prm.tiles_x * S.prm.tiles_y * S.prm.tiles_z;
     const size_t need = (size_t)ntiles * h->P * 3 * sizeof(double);
-    if (h->scratch_bytes < need) {
-        if (h->d_scratch) {
-            SAS_CUDA(cudaStreamSynchronize(st));
-            cudaFree(h->d_scratch);
-            h->d_scratch = nullptr;
-            h->scratch_bytes = 0;
-        }
-        SAS_CUDA(cudaMalloc(&h->d_scratch, need));
-        h->scratch_bytes = need;
-    }
+    void* part = nullptr;
+    bool own = false;
+    SAS_CUDA(call_scratch(h->partials, need, st, &part, &own));
     // (tile, ping) partials with no pair inside the beams are never written
-    SAS_CUDA(cudaMemsetAsync(h->d_scratch, 0, need, st));
+    cudaError_t e = cudaMemsetAsync(part, 0, need, st);
     S.prm.gimage = grad_image;
-    S.prm.partials = (double*)h->d_scratch;
-    rc = core::launch_mode<core::MODE_OFFSET_GRAD>(S, h->echo_dtype, dim3, st);
-    if (rc != SAS_OK) return rc;
-    const int n = h->P * 3;
-    core::reduce_tiles_kernel<<<(n + 31) / 32, 32 * core::RT_SLICES, 0, st>>>((const double*)h->d_scratch, (int)ntiles, n,
-                                                                 grad_offsets);
-    SAS_CUDA(cudaGetLastError());
-    return SAS_OK;
+    S.prm.partials = (double*)part;
+    rc = e == cudaSuccess ? core::launch_mode<core::MODE_OFFSET_GRAD>(S, h->echo_dtype, dim3, st)
+                          : cuda_fail(e, "offset gradient memset");
+    if (rc == SAS_OK) {
+        const int n = h->P * 3;
+        core::reduce_tiles_kernel<<<(n + 31) / 32, 32 * core::RT_SLICES, 0, st>>>((const double*)part, (int)ntiles, n,
+                                                                                 grad_offsets);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) rc = cuda_fail(e, "reduce_tiles_kernel");
+    }
+    if (own) cudaFreeAsync(part, st);
+    return rc;
 }
 
 }  // namespace sas
