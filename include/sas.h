@@ -192,7 +192,10 @@ int sas_geometry_destroy(sas_geometry_t h);
  * SAS_ECHO_C64 copies as is; the 16-bit types divide each (ping, channel) row
  * by its largest |component| (kept as a float32 scale and re-applied inside
  * the kernels) and round to float16 / bfloat16 on the device.  Replaces any
- * previous echo.  Errors: SAS_ERR_ARG, SAS_ERR_OOM, SAS_ERR_CUDA. */
+ * previous echo.  The first upload, and one of another size, allocates the
+ * storage (and 70 MB of scratch for the images, see sas_backproject_2d) and may
+ * wait for the stream; an upload of the same size from the device does neither.
+ * Errors: SAS_ERR_ARG, SAS_ERR_OOM, SAS_ERR_CUDA. */
 int sas_echo_upload(sas_geometry_t h, const void* echo, int on_device, int store_dtype,
                     void* cuda_stream);
 
@@ -204,8 +207,10 @@ int sas_echo_download(sas_geometry_t h, void* d_out, void* cuda_stream);
  * d_image: complex64 [ny][nx], device.  accumulate = 0 overwrites the image,
  * 1 adds to it (e.g. to stream pings through several echo uploads).
  * Small and middling grids are computed in several parts that are added in a fixed
- * order (the image does not depend on the run); the parts take up to 70 MB of scratch
- * that stays with the handle (stream-ordered memory while the stream is captured).
+ * order (the image does not depend on the run).  The parts lie in scratch that was reserved
+ * with the echo, so an image neither allocates device memory nor waits; where there was
+ * no memory to reserve, images are computed in one part.  While the stream is captured the
+ * graph owns its calls' scratch, here and in the offset gradient.
  * Errors: SAS_ERR_ARG, SAS_ERR_STATE (no echo), SAS_ERR_UNSUPPORTED (taps != 8,
  * a tile's delay span too long for the staging buffers), SAS_ERR_CUDA. */
 int sas_backproject_2d(sas_geometry_t h, const sas_grid* grid, const sas_interp* interp,

@@ -27,7 +27,7 @@ int cuda_fail(cudaError_t e, const char* what) {
     return e == cudaErrorMemoryAllocation ? SAS_ERR_OOM : SAS_ERR_CUDA;
 }
 
-cudaError_t call_scratch(HandleScratch& s, size_t bytes, cudaStream_t st, void** p, bool* own) {
+cudaError_t call_scratch(HandleScratch& s, size_t bytes, bool grow, cudaStream_t st, void** p, bool* own) {
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     *own = false;
     cudaError_t e = cudaStreamIsCapturing(st, &cs);
@@ -38,6 +38,7 @@ cudaError_t call_scratch(HandleScratch& s, size_t bytes, cudaStream_t st, void**
         return e;
     }
     if (s.bytes < bytes) {
+        if (!grow) return cudaErrorMemoryAllocation;
         if (s.p) {
             e = cudaStreamSynchronize(st);
             if (e != cudaSuccess) return e;
@@ -602,7 +603,8 @@ extern "C" int sas_echo_upload(sas_geometry_t h, const void* echo, int on_device
     const size_t rows = (size_t)h->P * h->C, Ns = h->Ns;
     const size_t elem = store_dtype == SAS_ECHO_C64 ? 8 : 4;
     const size_t need = rows * Ns * elem;
-    if (h->echo_bytes != need) {
+    const bool fresh = h->echo_bytes != need;
+    if (fresh) {
         if (h->d_echo) {
             SAS_CUDA(cudaStreamSynchronize(st));
             cudaFree(h->d_echo);
@@ -658,6 +660,8 @@ extern "C" int sas_echo_upload(sas_geometry_t h, const void* echo, int on_device
         if (rc != SAS_OK) return rc;
     }
     h->echo_dtype = store_dtype;
+    // here and not with the first image, so that images allocate nothing
+    if (fresh) reserve_planes(h, st);
     return SAS_OK;
 }
 

@@ -283,8 +283,8 @@ struct sas_geometry_s {
     float* d_scale;    // [P][C] (16-bit storage)
     int echo_dtype;    // -1 = none
     size_t echo_bytes;
-    // scratch, grown on demand: the offset gradient's partial sums, the forward pass's
-    // planes (two buffers, so that neither call's growth replaces the other's)
+    // scratch: the offset gradient's partial sums (grown on demand); the forward pass's
+    // planes (reserved with the echo, see reserve_planes)
     sas::HandleScratch partials, planes;
     // failure-detection test hook
     int debug_skip_copies;
@@ -318,10 +318,14 @@ int encode_echo_map(CUtensorMap* map, const void* base, int elem_bytes, int Ns, 
 
 int sm_count();
 
-// `bytes` of device memory for one call on `st`: the handle's buffer s, grown when it is
-// too small, or, while the stream is being captured, stream-ordered memory (*own: to be
-// freed on the stream after use) -- a graph must not keep a pointer that a later call of
-// the handle may replace.
-cudaError_t call_scratch(HandleScratch& s, size_t bytes, cudaStream_t st, void** p, bool* own);
+// `bytes` of device memory for one call on `st`: the handle's buffer s, grown (if `grow`)
+// when it is too small, or, while the stream is being captured, stream-ordered memory
+// (*own: to be freed on the stream after use) -- a graph must not keep a pointer that a
+// later call of the handle may replace.
+cudaError_t call_scratch(HandleScratch& s, size_t bytes, bool grow, cudaStream_t st, void** p, bool* own);
+
+// Reserves the planes of split images (launch_forward) for every grid, unless the stream
+// is being captured; without memory the handle's images run unsplit.
+void reserve_planes(sas_geometry_t h, cudaStream_t st);
 
 }  // namespace sas

@@ -8,6 +8,8 @@
 namespace sas {
 namespace core {
 
+constexpr int MAX_WAVES = 16;    // a split image takes at most so many waves of CTAs
+
 double series_range(sas_geometry_t h, double dmax, double ymax) {
     const double err_m = 5e-6 * h->sig.c / (2.0 * M_PI * std::max(std::fabs(h->sig.fc), h->sig.fs));
     return dmax + std::max(8.0 * ymax, std::pow(0.1 * std::pow(ymax, 5.0) / err_m, 0.25));
@@ -183,7 +185,7 @@ int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long slots, Setu
     // with 7 splits on the 304 slots of two CTAs an SM), 250 x 24 -> 1500 x 1101 in BF16 945
     // tiles on 304 (12.1 ms; 11.0 ms in splits).  Filling the pipeline and writing a
     // tile cost a CTA about 12 pairs' time.
-    prm.pings_per_split = slots > 0 ? pick_pings_per_split(ntiles, h->P, h->C, slots, 12.0, 16 * slots) : h->P;
+    prm.pings_per_split = slots > 0 ? pick_pings_per_split(ntiles, h->P, h->C, slots, 12.0, (long long)MAX_WAVES * slots) : h->P;
     const int nsplit = (h->P + prm.pings_per_split - 1) / prm.pings_per_split;
     prm.nsplit = nsplit;
     if (ntiles * nsplit > 0x7fffffffLL) {
@@ -253,6 +255,23 @@ __global__ void __launch_bounds__(256) sum_splits_kernel(const float2* __restric
 
 }  // namespace core
 
+void reserve_planes(sas_geometry_t h, cudaStream_t st) {
+    using namespace core;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (h->planes.p || h->P < 2 || cudaStreamIsCapturing(st, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone)
+        return;
+    // a split image's planes hold at most a tile for each of its CTAs: 70 MB
+    static_assert(Tile<false>::TX * Tile<false>::TY == NCONS * PX &&
+                  Tile<true>::TX * Tile<true>::TY * Tile<true>::TZ == NCONS * PX, "pixels of a tile");
+    const size_t bytes = sizeof(float2) * NCONS * PX * MAX_WAVES * 2 * sm_count();
+    if (cudaMalloc(&h->planes.p, bytes) == cudaSuccess) {
+        h->planes.bytes = bytes;
+    } else {
+        h->planes.p = nullptr;
+        (void)cudaGetLastError();
+    }
+}
+
 int launch_forward(const ForwardArgs& a) {
     core::Setup S;
     int rc = core::prepare(a.h, a.grid, a.dim3, 2LL * sm_count(), S);
@@ -266,7 +285,8 @@ int launch_forward(const ForwardArgs& a) {
     const size_t npix = (size_t)a.grid.nx * a.grid.ny * S.prm.nz;
     bool own = false;
     float2* parts = nullptr;
-    if (call_scratch(a.h->planes, sizeof(float2) * npix * S.prm.nsplit, a.stream, (void**)&parts, &own) != cudaSuccess) {
+    if (call_scratch(a.h->planes, sizeof(float2) * npix * S.prm.nsplit, false, a.stream, (void**)&parts, &own) !=
+        cudaSuccess) {
         (void)cudaGetLastError();   // no memory for the planes: one CTA a tile
         rc = core::prepare(a.h, a.grid, a.dim3, 0, S);
         if (rc != SAS_OK) return rc;

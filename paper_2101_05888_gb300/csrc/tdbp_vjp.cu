@@ -78,7 +78,7 @@ int launch_offset_grad(sas_geometry_t h, const sas_grid& g, const float2* grad_i
     const size_t need = (size_t)ntiles * h->P * 3 * sizeof(double);
     void* part = nullptr;
     bool own = false;
-    SAS_CUDA(call_scratch(h->partials, need, st, &part, &own));
+    SAS_CUDA(call_scratch(h->partials, need, true, st, &part, &own));
     // (tile, ping) partials with no pair inside the beams are never written
     cudaError_t e = cudaMemsetAsync(part, 0, need, st);
     S.prm.gimage = grad_image;

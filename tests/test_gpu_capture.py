@@ -59,3 +59,22 @@ def test_captured_gradient_and_image_survive_larger_calls():
         assert torch.equal(torch.view_as_real(again), torch.view_as_real(big0)) and torch.equal(big_grad, big_grad0)
     geom.sync_status()
     geom.close()
+
+
+@pytest.mark.parametrize("store", [sas.SAS_ECHO_C64, sas.SAS_ECHO_C32_BF16])
+def test_images_allocate_nothing(store):
+    """After the upload, images of growing size in plain calls (one part, many parts, a whole wave of
+    tiles) leave the free device memory as it is."""
+    geom, _ = _handle()
+    geom.upload_echo(synth.random_echo(48, 4, 1024, seed=94), store)
+    k = sas.kaiser(4.0)
+    sizes = [(1, 1), (60, 50), (300, 200), (900, 700), (1500, 1100), (2000, 1500)]
+    imgs = [torch.empty((1, ny, nx), dtype=torch.complex64, device="cuda") for nx, ny in sizes]
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    for (nx, ny), img in zip(sizes, imgs):
+        geom.backproject(sas.make_grid(1.0, 20.0, 0.0, 0.015, 0.015, 0.0, nx, ny), k, image=img)
+        torch.cuda.synchronize()
+        assert torch.cuda.mem_get_info()[0] == free
+    geom.sync_status()
+    geom.close()
