@@ -356,9 +356,11 @@ __device__ __forceinline__ PairGeoDF pair_geo_df(const KParams& p, const dfl* X0
 }
 // v != nullptr: the receiver's velocity during reception (Sec. II-D).  With beta = v / c
 // the two-way path s = c tau of the tile centre solves (s - |R_T|)^2 = |R_R - beta s|^2,
-//   s = (|R_T| - rho + sqrt((|R_T| - rho)^2 - (1 - beta^2)(|R_T|^2 - |R_R|^2))) / (1 - beta^2),
-// rho = R_R . beta, and R_R is then taken from the receiver's position at that time (an FP64
-// fixed point in its place kept the producer warp on the slow FP64 pipe: the stripmap
+//   s = (|R_T| - rho + sqrt(|W|^2 - (beta^2 |R_R|^2 - rho^2))) / (1 - beta^2),
+// W = R_R - beta |R_T|, rho = R_R . beta (the root's argument without the cancellation
+// of |R_T|^2 against |R_R|^2: s to 5e-12 m at 100 m, for any |beta| < 1 and down to a receiver
+// at the tile centre), and R_R is then taken from the receiver's position at that time (an
+// FP64 fixed point in its place kept the producer warp on the slow FP64 pipe: the stripmap
 // with motion ran at 0.76 of its rate without).
 __device__ __forceinline__ int pair_record_df(const KParams& p, PairGeoDF G, float* rc, int stride,
                                               const double* v = nullptr) {
@@ -374,12 +376,14 @@ __device__ __forceinline__ int pair_record_df(const KParams& p, PairGeoDF G, flo
         auto dot = [](const dfl* x, const dfl* y) {
             return df_add(df_add(df_mul(x[0], y[0]), df_mul(x[1], y[1])), df_mul(x[2], y[2]));
         };
-        const dfl one{1.0f, 0.0f}, b2 = dot(b, b), rho = dot(G.R, b), T2 = dot(G.T, G.T), R2 = dot(G.R, G.R);
-        const dfl m = df_add(df_sqrt(T2), df_neg(rho));
-        const dfl disc = df_add(df_mul(m, m), df_neg(df_mul(df_add(one, df_neg(b2)), df_add(T2, df_neg(R2)))));
-        // 1 / (1 - beta^2) = 1 + beta^2 + beta^4 (beta^6 ~ 1e-18)
-        const dfl inv = df_add(one, df_add(b2, df_mul(b2, b2)));
-        const dfl s = df_mul(df_add(m, df_sqrt(disc)), inv);
+        const dfl b2 = dot(b, b), rho = dot(G.R, b), n = df_sqrt(dot(G.T, G.T));
+        dfl W[3];
+#pragma unroll
+        for (int k = 0; k < 3; ++k) W[k] = df_add(G.R[k], df_neg(df_mul(b[k], n)));
+        dfl disc = df_add(dot(W, W), df_add(df_mul(rho, rho), df_neg(df_mul(b2, dot(G.R, G.R)))));
+        if (disc.hi <= 0.0f) disc = dfl{0.0f, 0.0f};   // zero but for rounding
+        const dfl s = df_mul(df_add(df_add(n, df_neg(rho)), df_sqrt(disc)),
+                             df_recip(df_add(dfl{1.0f, 0.0f}, df_neg(b2))));
 #pragma unroll
         for (int k = 0; k < 3; ++k) G.R[k] = df_add(G.R[k], df_neg(df_mul(b[k], s)));
         rc[F_RV * stride] = df_float(dot(G.R, b));
