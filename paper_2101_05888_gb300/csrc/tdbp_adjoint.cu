@@ -101,21 +101,19 @@ __global__ void __launch_bounds__(NTHREADS, 2) adjoint_kernel(const KParams p, c
         __syncthreads();   // previous stage's records no longer in use
         if (warp == 0 && qs + lane < q1) {
             const int i = (int)((unsigned)(qs + lane) / (unsigned)p.C);
-            // the forward pass's reference terms: double-float for stop-and-hop, FP64 with
-            // motion or refraction
+            // the forward pass's reference terms (beam decisions agree bit for bit):
+            // double-float for straight legs, FP64 with refraction
             if (REFRACT) {
                 const PairGeo G = pair_geo(p, X0, Y0, Z0, qs + lane, i);
                 double LT0, LR0;
                 rfl_s[lane] = refr_pair_blocks(p, G, p.tx[3 * (size_t)i + 2], p.rx[3 * (size_t)(qs + lane) + 2], bmask,
                                                Zr, Z0, rec + lane, PAIRS, LT0, LR0);
-                base_s[lane] = pair_record(p, G, rec + lane, PAIRS, nullptr, LT0, LR0);
-            } else if (p.vel) {
-                base_s[lane] = pair_record(p, pair_geo(p, X0, Y0, Z0, qs + lane, i), rec + lane, PAIRS,
-                                           p.vel + 3 * (size_t)i);
+                base_s[lane] = pair_record(p, G, rec + lane, PAIRS, LT0, LR0);
             } else {
                 const float2 a = df_split(X0), b = df_split(Y0), c = df_split(Z0);
                 const dfl X0d[3] = {dfl{a.x, a.y}, dfl{b.x, b.y}, dfl{c.x, c.y}};
-                base_s[lane] = pair_record_df(p, pair_geo_df(p, X0d, (int)(qs + lane), i), rec + lane, PAIRS);
+                base_s[lane] = pair_record_df(p, pair_geo_df(p, X0d, (int)(qs + lane), i), rec + lane, PAIRS,
+                                              p.vel ? p.vel + 3 * (size_t)i : nullptr);
             }
         }
         __syncthreads();

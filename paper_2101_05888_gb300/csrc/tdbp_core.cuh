@@ -273,7 +273,7 @@ __device__ __forceinline__ PairGeo pair_geo(const KParams& p, double X0, double 
     return PairGeo{X0 - t[0], Y0 - t[1], Z0 - t[2], X0 - r[0], Y0 - r[1], Z0 - r[2]};
 }
 
-// FP64 reference terms of a pair written to the record rc (field f at
+// FP64 reference terms of a pair (seabed refraction) written to the record rc (field f at
 // rc[f * stride]): 2R and |R|^2, |R| for transmitter and receiver, twice the
 // fraction of u_ref = (tau_ref - t0) fs minus 1/2 (so that rounding
 // 2(u - floor u_ref) - 1/2 to the nearest integer gives the half-sample index
@@ -282,35 +282,10 @@ __device__ __forceinline__ PairGeo pair_geo(const KParams& p, double X0, double 
 // Returns the raw sample index of Farrow position 0, tap 0: floor(u_ref) - U - 3.
 // LT0, LR0 >= 0: leg lengths at x0 in water metres (seabed refraction) that
 // replace |R_T|, |R_R| in tau_ref; the differential fields stay the straight ones.
-__device__ __forceinline__ int pair_record(const KParams& p, PairGeo G, float* rc, int stride, const double* v,
-                                           double LT0 = -1.0, double LR0 = -1.0) {
+__device__ __forceinline__ int pair_record(const KParams& p, const PairGeo& G, float* rc, int stride, double LT0,
+                                           double LR0) {
     const double nT2 = G.Tx * G.Tx + G.Ty * G.Ty + G.Tz * G.Tz;
     const double nT = sqrt(nT2);
-    if (v) {
-        // receiver moving during reception (Sec. II-D): the tile centre's
-        // echo arrives at tau with c tau = |R_T| + |R_R - v tau|; fixed-point
-        // iteration (contraction |v|/c), then R_R from the receiver's position
-        // at that time
-        const double vx = v[0], vy = v[1], vz = v[2];
-        rc[F_BRX * stride] = (float)(2.0 * G.Rx);
-        rc[F_BRY * stride] = (float)(2.0 * G.Ry);
-        rc[F_BRZ * stride] = (float)(2.0 * G.Rz);
-        double tau = (nT + sqrt(G.Rx * G.Rx + G.Ry * G.Ry + G.Rz * G.Rz)) * p.inv_c;
-        for (int it = 0; it < 12; ++it) {
-            const double wx = G.Rx - vx * tau, wy = G.Ry - vy * tau, wz = G.Rz - vz * tau;
-            const double t2 = (nT + sqrt(wx * wx + wy * wy + wz * wz)) * p.inv_c;
-            const double step = fabs(t2 - tau);
-            tau = t2;
-            if (step <= 1e-16 * tau) break;
-        }
-        G.Rx -= vx * tau;
-        G.Ry -= vy * tau;
-        G.Rz -= vz * tau;
-        rc[F_VX * stride] = (float)(vx * p.inv_c);
-        rc[F_VY * stride] = (float)(vy * p.inv_c);
-        rc[F_VZ * stride] = (float)(vz * p.inv_c);
-        rc[F_RV * stride] = (float)((G.Rx * vx + G.Ry * vy + G.Rz * vz) * p.inv_c);
-    }
     const double nR2 = G.Rx * G.Rx + G.Ry * G.Ry + G.Rz * G.Rz;
     const double nR = sqrt(nR2);
     const double tau = ((LT0 >= 0.0 ? LT0 : nT) + (LR0 >= 0.0 ? LR0 : nR)) * p.inv_c;
@@ -334,8 +309,8 @@ __device__ __forceinline__ int pair_record(const KParams& p, PairGeo G, float* r
     return (int)iref - p.U - 3;
 }
 
-// The same pair vectors and reference terms in double-float arithmetic (the
-// stop-and-hop model with straight legs): R = x0 - sensor to about 48 bits,
+// The same pair vectors and reference terms in double-float arithmetic
+// (straight legs): R = x0 - sensor to about 48 bits,
 // |R|^2 and |R| (|R| to a few units of 2^-45 relative), the two-way path, u_ref
 // and the carrier phase.  The outputs are the FP32 fields pair_record writes;
 // the phase and the fraction of u_ref keep about 1e-10 of a cycle / sample.
@@ -1029,7 +1004,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
                     if constexpr (DFREC)
                         base = pair_record_df(p, Gd, rc, 1, MOTION ? p.vel + 3 * (size_t)iv : nullptr);
                     else
-                        base = pair_record(p, Gv, rc, 1, nullptr, LT0, LR0);
+                        base = pair_record(p, Gv, rc, 1, LT0, LR0);
                     const int seg_start = base - (((base % p.seg_align) + p.seg_align) % p.seg_align);
                     rc[F_OFF] = __int_as_float(base - seg_start);
                     rc[F_SCALE] = p.scale ? p.scale[qv] : 1.0f;

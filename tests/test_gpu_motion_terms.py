@@ -66,3 +66,30 @@ def test_receiver_at_a_tile_centre(moving):
     # first order in that against the range: pixels beyond 0.2 m, to 0.42 rad x (5e-3 / 0.2)^2
     far = np.linalg.norm(pix - centre, axis=1).reshape(img.shape) > 0.2
     assert oracle.rel_l2(img[far], ref[far]) < 3e-4
+
+
+@pytest.mark.parametrize("speed", [1.95, 60.0])
+def test_adjoint_takes_the_forward_terms_with_beam_and_motion(speed):
+    """<B e, G> = <e, B^H G> over a grid that beam edges sweep across: both passes form
+    the same reference terms, so they take the same decisions and delays (one term
+    decided differently moves the product by about 1; FP32 rounding by ~1e-6 of a random
+    inner product's size, as in the dot test of the beam alone)."""
+    g = synth.Grid(8.0, 40.0, 0.0, 0.03, 0.03, 0.0, 160, 60, 1)
+    w = synth.workload("stripmap_2d", grid=g, n_pings=40, n_rx=2, n_samples=4096, t0=0.05)
+    nav = synth.nav(w)
+    geom = sas.Geometry.from_nav(nav, lib_signal(w))
+    geom.set_beam(np.deg2rad(25.0), 1)
+    geom.set_velocity(np.tile(speed * np.array([1.0, 0.02, -0.01]), (40, 1)))
+    echo = synth.random_echo(40, 2, 4096, seed=103)
+    geom.upload_echo(echo)
+    G = synth.random_image((1, g.ny, g.nx), seed=104).astype(np.complex64)
+    eadj = torch.empty((40, 2, 4096), dtype=torch.complex64, device="cuda")
+    Be = geom.backproject(sas.grid_from(g), sas.kaiser(4.0)).cpu().numpy().reshape(-1).astype(np.complex128)
+    sas.sas_backproject_adjoint(geom.h, sas.grid_from(g), sas.kaiser(4.0), torch.from_numpy(G).cuda(), eadj)
+    geom.sync_status()
+    geom.close()
+    Gv = G.reshape(-1).astype(np.complex128)
+    lhs = np.vdot(Be, Gv)
+    rhs = np.vdot(echo.reshape(-1).astype(np.complex128), eadj.cpu().numpy().reshape(-1).astype(np.complex128))
+    print("speed %g: %.2e" % (speed, abs(lhs - rhs) / (np.linalg.norm(Be) * np.linalg.norm(Gv) / np.sqrt(Gv.size))))
+    assert abs(lhs - rhs) <= 2e-5 * np.linalg.norm(Be) * np.linalg.norm(Gv) / np.sqrt(Gv.size)
