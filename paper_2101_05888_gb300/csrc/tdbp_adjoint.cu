@@ -639,7 +639,7 @@ static bool adjoint2d_plan(sas_geometry_t h, const sas_grid& g, core::Setup& S, 
     p.tiles_y = (g.ny + AT - 1) / AT;
     // (loading a tile and clearing the rows costs about four pairs' time)
     const long long ntiles = (long long)p.tiles_x * p.tiles_y;
-    p.pings_per_split = pick_pings_per_split(ntiles, h->P, h->C, 2LL * sm_count(), 4.0, 4864);
+    p.pings_per_split = pick_pings_per_split(ntiles, h->P, h->C, 2LL * sm_count(), false, 4.0, 0.0, 4864);
     p.nsplit = (h->P + p.pings_per_split - 1) / p.pings_per_split;
     S.blocks = (int)(ntiles * p.nsplit);
     return true;

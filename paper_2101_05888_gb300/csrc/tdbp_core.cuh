@@ -1781,10 +1781,12 @@ inline void tile_dims(int dim3, int& TXs, int& TYs, int& TZs) {
 double series_range(sas_geometry_t h, double dmax, double ymax);
 
 // Pings per block when `ntiles` tiles of P pings x C channels run on `slots`
-// resident blocks: the split with the least time in whole waves of blocks, where a
-// block costs its pairs plus `overhead` pairs; at most max_blocks blocks (or
-// one a tile).
-int pick_pings_per_split(long long ntiles, int P, int C, long long slots, double overhead, long long max_blocks);
+// resident blocks: the split with the least time, where a block costs its pairs plus
+// `overhead` pairs, the blocks run in whole waves (uneven: blocks of unequal work run one after
+// another on each slot, and the last one takes a block's time), and a split launch costs
+// `sum_cost` pairs more; at most max_blocks blocks (or one a tile).
+int pick_pings_per_split(long long ntiles, int P, int C, long long slots, bool uneven, double overhead,
+                         double sum_cost, long long max_blocks);
 
 int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long slots, Setup& S, bool need_echo = true,
             int mode = MODE_FORWARD);

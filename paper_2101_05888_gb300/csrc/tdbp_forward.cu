@@ -15,17 +15,23 @@ double series_range(sas_geometry_t h, double dmax, double ymax) {
     return dmax + std::max(8.0 * ymax, std::pow(0.1 * std::pow(ymax, 5.0) / err_m, 0.25));
 }
 
-int pick_pings_per_split(long long ntiles, int P, int C, long long slots, double overhead, long long max_blocks) {
+int pick_pings_per_split(long long ntiles, int P, int C, long long slots, bool uneven, double overhead,
+                         double sum_cost, long long max_blocks) {
     int best = P;
     double best_cost = 0.0;
-    for (long long s = 1; s <= P && (s == 1 || s * ntiles <= max_blocks); ++s) {
-        const int pps = (int)((P + s - 1) / s);
-        const long long blocks = ntiles * ((P + pps - 1) / pps);
-        const double cost = (double)((blocks + slots - 1) / slots) * ((double)pps * C + overhead);
+    const double per_slot = (double)ntiles / (double)slots;
+    for (int s = 1; s <= P && (s == 1 || s * ntiles <= max_blocks);) {
+        // not below this for s splits or more: every slot's share of the pairs and of the overheads
+        if (s > 1 && per_slot * ((double)P * C + s * overhead) >= best_cost) break;
+        const int pps = (P + s - 1) / s, nsplit = (P + pps - 1) / pps;
+        const double waves = uneven ? per_slot * nsplit + 1.0 : std::ceil(per_slot * nsplit - 1e-9);
+        const double cost = waves * ((double)pps * C + overhead) + (s > 1 ? sum_cost : 0.0);
         if (s == 1 || cost < best_cost) {
             best_cost = cost;
             best = pps;
         }
+        if (pps == 1) break;
+        s = (P - 1) / (pps - 1) + 1;   // the next split with fewer pings a block
     }
     return best;
 }
@@ -184,8 +190,14 @@ int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long slots, Setu
     // of CTAs: 128 pings x 4 RX -> 256^2 at 2 cm ran 320 CTAs on 152 slots (129 us a call; 84 us
     // with 7 splits on the 304 slots of two CTAs an SM), 250 x 24 -> 1500 x 1101 in BF16 945
     // tiles on 304 (12.1 ms; 11.0 ms in splits).  Filling the pipeline and writing a
-    // tile cost a CTA about 12 pairs' time.
-    prm.pings_per_split = slots > 0 ? pick_pings_per_split(ntiles, h->P, h->C, slots, 12.0, (long long)MAX_WAVES * slots) : h->P;
+    // tile cost a CTA about 12 pairs' time; adding the parts is another launch, five pairs'
+    // time (3 pings x 2 RX -> one tile: 10.0 us in one part, 11.3 us in three).  With a
+    // beam the CTAs compute between none and all of their pairs, so whole waves mean
+    // nothing (150 x 4 -> 400 x 300 at 3 cm, 30 degrees: 288 us by whole waves, 257 us now).
+    const double sum_cost = mode == MODE_FORWARD && need_echo ? 5.0 : 0.0;
+    prm.pings_per_split = slots > 0 ? pick_pings_per_split(ntiles, h->P, h->C, slots, prm.beam, 12.0, sum_cost,
+                                                           (long long)MAX_WAVES * slots)
+                                    : h->P;
     const int nsplit = (h->P + prm.pings_per_split - 1) / prm.pings_per_split;
     prm.nsplit = nsplit;
     if (ntiles * nsplit > 0x7fffffffLL) {
@@ -242,15 +254,45 @@ int launch_mode(const Setup& S, int echo_dtype, int dim3, cudaStream_t st) {
 
 template int launch_mode<MODE_FORWARD>(const Setup&, int, int, cudaStream_t);
 
-// image = (accumulate ? image : 0) + the parts in order
+// image = (accumulate ? image : 0) + the parts in a fixed order.  SLICES threads a pixel,
+// each over every SLICES-th part, four loads in flight: with one thread a pixel 300 parts of a
+// single tile took 20 us, one load after the other.
+template <int SLICES>
 __global__ void __launch_bounds__(256) sum_splits_kernel(const float2* __restrict__ parts, size_t npix, int nsplit,
                                                          int accumulate, float2* __restrict__ image) {
-    const size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x;
-    if (i >= npix) return;
-    float2 s = parts[i];
-    for (int k = 1; k < nsplit; ++k) s = fadd2(s, parts[k * npix + i]);
-    if (accumulate) s = fadd2(s, image[i]);
-    image[i] = s;
+    constexpr int W = 256 / SLICES;
+    __shared__ float2 red[SLICES][W];
+    const int x = threadIdx.x % W, sl = threadIdx.x / W;
+    const size_t i = blockIdx.x * (size_t)W + x;
+    float2 s = make_float2(0.f, 0.f);
+    if (i < npix) {
+        int k = sl;
+        for (; k + 3 * SLICES < nsplit; k += 4 * SLICES) {
+            float2 v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = parts[(k + u * SLICES) * npix + i];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) s = fadd2(s, v[u]);
+        }
+        for (; k < nsplit; k += SLICES) s = fadd2(s, parts[k * npix + i]);
+    }
+    if (SLICES > 1) {
+        red[sl][x] = s;
+        __syncthreads();
+        if (sl == 0)
+            for (int t = 1; t < SLICES; ++t) s = fadd2(s, red[t][x]);
+    }
+    if (sl == 0 && i < npix) {
+        if (accumulate) s = fadd2(s, image[i]);
+        image[i] = s;
+    }
+}
+
+void sum_splits(const float2* parts, size_t npix, int nsplit, int accumulate, float2* image, cudaStream_t st) {
+    if (nsplit >= 16)
+        sum_splits_kernel<8><<<(unsigned)((npix + 31) / 32), 256, 0, st>>>(parts, npix, nsplit, accumulate, image);
+    else
+        sum_splits_kernel<1><<<(unsigned)((npix + 255) / 256), 256, 0, st>>>(parts, npix, nsplit, accumulate, image);
 }
 
 }  // namespace core
@@ -299,8 +341,7 @@ int launch_forward(const ForwardArgs& a) {
     S.prm.accumulate = 0;
     rc = core::launch_mode<core::MODE_FORWARD>(S, a.h->echo_dtype, a.dim3, a.stream);
     if (rc == SAS_OK) {
-        core::sum_splits_kernel<<<(unsigned)((npix + 255) / 256), 256, 0, a.stream>>>(parts, npix, S.prm.nsplit,
-                                                                                     a.accumulate, a.image);
+        core::sum_splits(parts, npix, S.prm.nsplit, a.accumulate, a.image, a.stream);
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) rc = cuda_fail(e, "sum_splits_kernel");
     }
