@@ -111,45 +111,59 @@ int encode_echo_map(CUtensorMap* map, const void* base, int elem_bytes, int Ns, 
 // ---------------------------------------------------------------------------
 // Sensor positions (Sec. II-C): x_TX,i = p_i + dp_i + R_i l_TX, x_RX,i,c = p_i + dp_i + R_i l_c,
 // with R_i the attitude rotation of Eq. 2 (attitude_rotation).
-// One warp a ping: three lanes take the angles' sines and cosines, then a lane a
-// sensor (a thread a ping took 24 us for 256 pings x 16 receivers, one long chain of FP64
-// operations; autofocus moves the sensors twice a step).
-constexpr int GEO_WARPS = 4;
-__global__ void __launch_bounds__(32 * GEO_WARPS) geometry_kernel(int P, int C, const double* __restrict__ pos, const double* __restrict__ att,
-                                const double* __restrict__ lever, const double* __restrict__ off,
-                                double* __restrict__ tx, double* __restrict__ rx, float* __restrict__ rotc,
-                                float2* __restrict__ txs, float2* __restrict__ rxs) {
-    const int i = blockIdx.x * GEO_WARPS + (threadIdx.x >> 5), lane = threadIdx.x & 31;
-    if (i >= P) return;   // whole warps
-    double R[9], sn, cs;
-    sincos(att[3 * i + lane % 3], &sn, &cs);
-    rotation_of(__shfl_sync(0xffffffffu, sn, 0), __shfl_sync(0xffffffffu, cs, 0), __shfl_sync(0xffffffffu, sn, 1),
-                __shfl_sync(0xffffffffu, cs, 1), __shfl_sync(0xffffffffu, sn, 2), __shfl_sync(0xffffffffu, cs, 2), R);
-    const double b0 = pos[3 * i] + off[3 * i], b1 = pos[3 * i + 1] + off[3 * i + 1],
-                 b2 = pos[3 * i + 2] + off[3 * i + 2];
-    // columns 0 and 1 of R: body-frame components (R^T v).x, (R^T v).y of a NED vector v
-    if (lane == 0) {
-        rotc[6 * i + 0] = (float)R[0];
-        rotc[6 * i + 1] = (float)R[3];
-        rotc[6 * i + 2] = (float)R[6];
-        rotc[6 * i + 3] = (float)R[1];
-        rotc[6 * i + 4] = (float)R[4];
-        rotc[6 * i + 5] = (float)R[7];
+// A block takes `per` pings: a thread an angle for the sines and cosines, a thread a ping for
+// its rotation, then a thread a sensor.  Bound by latency at a few pings (8 a block) and by
+// the FP64 pipe at many (32 a block, so that the first two phases fill their warps): a
+// thread a ping over all its sensors took 24 us for 256 pings x 16 receivers (and 1.6 ms for
+// one ping of 2000, now 24 us), a warp a ping, its 32 lanes repeating three angles, 215 us
+// for 50000 x 8 (now 42 us).  Autofocus moves the sensors twice a step.
+constexpr int GEO_P = 32, GEO_T = 128;
+__global__ void __launch_bounds__(GEO_T) geometry_kernel(int P, int C, int per, const double* __restrict__ pos,
+                                                         const double* __restrict__ att,
+                                                         const double* __restrict__ lever,
+                                                         const double* __restrict__ off, double* __restrict__ tx,
+                                                         double* __restrict__ rx, float* __restrict__ rotc,
+                                                         float2* __restrict__ txs, float2* __restrict__ rxs) {
+    __shared__ double sc[GEO_P][6], rot[GEO_P][9], base[GEO_P][3];
+    const int i0 = blockIdx.x * per, np = min(per, P - i0), tid = threadIdx.x;
+    if (tid < 3 * np) {
+        const int j = tid / 3, a = tid % 3;
+        sincos(att[3 * (size_t)i0 + tid], &sc[j][2 * a], &sc[j][2 * a + 1]);
+        base[j][a] = pos[3 * (size_t)i0 + tid] + off[3 * (size_t)i0 + tid];
     }
-    for (int c = lane - 1; c < C; c += 32) {
-        const double* l = lever + 3 * (c + 1);
-        double* o = (c < 0) ? tx + 3 * (size_t)i : rx + 3 * ((size_t)i * C + c);
-        o[0] = b0 + R[0] * l[0] + R[1] * l[1] + R[2] * l[2];
-        o[1] = b1 + R[3] * l[0] + R[4] * l[1] + R[5] * l[2];
-        o[2] = b2 + R[6] * l[0] + R[7] * l[1] + R[8] * l[2];
-        float2* os = (c < 0) ? txs + 3 * (size_t)i : rxs + 3 * ((size_t)i * C + c);
+    __syncthreads();
+    if (tid < np) {
+        const double* s = sc[tid];
+        double* R = rot[tid];
+        rotation_of(s[0], s[1], s[2], s[3], s[4], s[5], R);
+        // columns 0 and 1 of R: body-frame components (R^T v).x, (R^T v).y of a NED vector v
+        float* o = rotc + 6 * (size_t)(i0 + tid);
+        o[0] = (float)R[0];
+        o[1] = (float)R[3];
+        o[2] = (float)R[6];
+        o[3] = (float)R[1];
+        o[4] = (float)R[4];
+        o[5] = (float)R[7];
+    }
+    __syncthreads();
+    for (int e = tid; e < np * (C + 1); e += GEO_T) {
+        const int j = e / (C + 1), c = e - j * (C + 1) - 1;
+        const size_t i = (size_t)(i0 + j);
+        const double *R = rot[j], *l = lever + 3 * (size_t)(c + 1);
+        const size_t at = c < 0 ? 3 * i : 3 * (i * C + c);
+        double* o = (c < 0 ? tx : rx) + at;
+        o[0] = base[j][0] + R[0] * l[0] + R[1] * l[1] + R[2] * l[2];
+        o[1] = base[j][1] + R[3] * l[0] + R[4] * l[1] + R[5] * l[2];
+        o[2] = base[j][2] + R[6] * l[0] + R[7] * l[1] + R[8] * l[2];
+        float2* os = (c < 0 ? txs : rxs) + at;
         for (int k = 0; k < 3; ++k) os[k] = df_split(o[k]);
     }
 }
 
 static int run_geometry(sas_geometry_t h, cudaStream_t st) {
-    geometry_kernel<<<(h->P + GEO_WARPS - 1) / GEO_WARPS, 32 * GEO_WARPS, 0, st>>>(h->P, h->C, h->d_pos, h->d_att, h->d_lever, h->d_off,
-                                                        h->d_tx, h->d_rx, h->d_rotc, h->d_txs, h->d_rxs);
+    const int per = h->P >= 8192 ? GEO_P : 8;
+    geometry_kernel<<<(h->P + per - 1) / per, GEO_T, 0, st>>>(h->P, h->C, per, h->d_pos, h->d_att, h->d_lever, h->d_off,
+                                                              h->d_tx, h->d_rx, h->d_rotc, h->d_txs, h->d_rxs);
     SAS_CUDA(cudaGetLastError());
     return SAS_OK;
 }
