@@ -973,8 +973,13 @@ extern "C" int sas_matched_filter(const void* d_raw, int64_t rows, int32_t n, co
     }
     const int M = NF - L + 1;
     const int nblk = (int)((n + M - 1) / M);
+    // in place, a row of several blocks is read from a copy, a run of rows at a time: a
+    // block's input reaches L - 1 samples into the next block's outputs, and the blocks of
+    // a row run at the same time
+    const bool copied = d_out == d_raw && nblk > 1;
+    const int64_t run = copied ? std::min<int64_t>(rows, std::max<int64_t>(1, ((int64_t)64 << 20) / ((int64_t)n * 8))) : rows;
     float2* Pc = nullptr;
-    SAS_CUDA(cudaMallocAsync((void**)&Pc, sizeof(float2) * NF, st));
+    SAS_CUDA(cudaMallocAsync((void**)&Pc, sizeof(float2) * (NF + (copied ? (size_t)run * n : 0)), st));
     const int nt = fft_threads(NF);
     const size_t sm = sizeof(float2) * (NF + NF / 2);       // row + twiddles
     int rc = SAS_OK;
@@ -983,17 +988,22 @@ extern "C" int sas_matched_filter(const void* d_raw, int64_t rows, int32_t n, co
         mf_replica_kernel<<<1, nt, sm, st>>>((const float2*)d_replica, L, NF, Pc);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) {
-        const float2* raw = (const float2*)d_raw;
-        float2* o = (float2*)d_out;
-        switch (NF) {
-            case 256: e = mf_reg_launch<256>(raw, rows, n, M, nblk, Pc, o, st); break;
-            case 512: e = mf_reg_launch<512>(raw, rows, n, M, nblk, Pc, o, st); break;
-            case 1024: e = mf_reg_launch<1024>(raw, rows, n, M, nblk, Pc, o, st); break;
-            case 2048: e = mf_reg_launch<2048>(raw, rows, n, M, nblk, Pc, o, st); break;
-            case 4096: e = mf_reg_launch<4096>(raw, rows, n, M, nblk, Pc, o, st); break;
-            case 8192: e = mf_reg_launch<8192>(raw, rows, n, M, nblk, Pc, o, st); break;
-            default: e = mf_reg_launch<16384>(raw, rows, n, M, nblk, Pc, o, st); break;
+    for (int64_t r0 = 0; r0 < rows && e == cudaSuccess; r0 += run) {
+        const int64_t nr = std::min(run, rows - r0);
+        const float2* raw = (const float2*)d_raw + r0 * n;
+        float2* o = (float2*)d_out + r0 * n;
+        if (copied) {
+            e = cudaMemcpyAsync(Pc + NF, raw, sizeof(float2) * (size_t)nr * n, cudaMemcpyDeviceToDevice, st);
+            raw = Pc + NF;
+        }
+        if (e == cudaSuccess) switch (NF) {
+            case 256: e = mf_reg_launch<256>(raw, nr, n, M, nblk, Pc, o, st); break;
+            case 512: e = mf_reg_launch<512>(raw, nr, n, M, nblk, Pc, o, st); break;
+            case 1024: e = mf_reg_launch<1024>(raw, nr, n, M, nblk, Pc, o, st); break;
+            case 2048: e = mf_reg_launch<2048>(raw, nr, n, M, nblk, Pc, o, st); break;
+            case 4096: e = mf_reg_launch<4096>(raw, nr, n, M, nblk, Pc, o, st); break;
+            case 8192: e = mf_reg_launch<8192>(raw, nr, n, M, nblk, Pc, o, st); break;
+            default: e = mf_reg_launch<16384>(raw, nr, n, M, nblk, Pc, o, st); break;
         }
     }
     if (e != cudaSuccess) rc = cuda_fail(e, "matched filter");
