@@ -1075,22 +1075,32 @@ extern "C" int sas_tvg(const void* d_in, void* d_out, int64_t rows, int32_t n, d
         return SAS_ERR_ARG;
     }
     cudaStream_t st = (cudaStream_t)stream;
-    double* med = d_median;
-    double* own = nullptr;
-    float* gain = d_gain;
-    if (!med || !gain) {
-        SAS_CUDA(cudaMallocAsync((void**)&own, sizeof(double) * n + sizeof(float) * n, st));
-        if (!med) med = own;
-        if (!gain) gain = reinterpret_cast<float*>(own + n);
+    // one allocation: the median and gain the caller does not ask for, and the bracketed
+    // select's brackets, candidates, counts and flags.  Without memory for the latter the
+    // three-level select runs, which needs none.
+    auto up256 = [](size_t x) { return (x + 255) / 256 * 256; };
+    const size_t own_bytes = d_median && d_gain ? 0 : up256((sizeof(double) + sizeof(float)) * (size_t)n);
+    const size_t o_c = own_bytes + up256(sizeof(uint2) * (size_t)n);
+    const size_t o_b = o_c + sizeof(unsigned) * (size_t)n * TVG_CAP;
+    const size_t o_n = o_b + sizeof(unsigned) * n, o_f = o_n + sizeof(unsigned) * n;
+    bool bracketed = rows >= TVG_BRACKET_MIN_ROWS;
+    char* scr = nullptr;
+    if (bracketed && cudaMallocAsync((void**)&scr, o_f + sizeof(int) * n, st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        bracketed = false;
+        scr = nullptr;
     }
+    if (!bracketed && own_bytes) SAS_CUDA(cudaMallocAsync((void**)&scr, own_bytes, st));
+    double* med = d_median ? d_median : reinterpret_cast<double*>(scr);
+    float* gain = d_gain ? d_gain : reinterpret_cast<float*>(scr + sizeof(double) * n);
     cudaError_t e0 = cudaFuncSetAttribute(tvg_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TVG_SMEM);
     if (e0 != cudaSuccess) {
-        if (own) cudaFreeAsync(own, st);
+        if (scr) cudaFreeAsync(scr, st);
         return cuda_fail(e0, "tvg");
     }
     const unsigned strips = (unsigned)((n + TVG_COLS - 1) / TVG_COLS);
     const float2* ein = (const float2*)d_in;
-    if (rows < TVG_BRACKET_MIN_ROWS) {
+    if (!bracketed) {
         tvg_select_kernel<<<strips, TVG_THREADS, TVG_SMEM, st>>>(ein, rows, 1, n, (unsigned)((rows - 1) / 2),
                                                                  (unsigned)(rows / 2), med, nullptr);
     } else {
@@ -1098,17 +1108,7 @@ extern "C" int sas_tvg(const void* d_in, void* d_out, int64_t rows, int32_t n, d
         const long long rstep = rows / (rows < TVG_FEW_ROWS ? TVG_SAMPLE_FEW : TVG_SAMPLE), m = (rows + rstep - 1) / rstep;
         const long long d = (long long)std::ceil(2.0 * std::sqrt((double)m)) + 1;
         const unsigned k_lo = (unsigned)std::max(0LL, (m - 1) / 2 - d), k_hi = (unsigned)std::min(m - 1, m / 2 + d);
-        // scratch: brackets, candidates, counts, flags
-        const size_t o_c = (sizeof(uint2) * n + 255) / 256 * 256;
-        const size_t o_b = o_c + sizeof(unsigned) * (size_t)n * TVG_CAP;
-        const size_t o_n = o_b + sizeof(unsigned) * n, o_f = o_n + sizeof(unsigned) * n;
-        char* scr = nullptr;
-        cudaError_t ea = cudaMallocAsync((void**)&scr, o_f + sizeof(int) * n, st);
-        if (ea != cudaSuccess) {
-            if (own) cudaFreeAsync(own, st);
-            return cuda_fail(ea, "tvg scratch");
-        }
-        uint2* br = reinterpret_cast<uint2*>(scr);
+        uint2* br = reinterpret_cast<uint2*>(scr + own_bytes);
         unsigned* cand = reinterpret_cast<unsigned*>(scr + o_c);
         unsigned* nb = reinterpret_cast<unsigned*>(scr + o_b);
         unsigned* ni = reinterpret_cast<unsigned*>(scr + o_n);
@@ -1117,14 +1117,13 @@ extern "C" int sas_tvg(const void* d_in, void* d_out, int64_t rows, int32_t n, d
         tvg_collect_kernel<<<strips, TVG_THREADS, 0, st>>>(ein, rows, n, br, cand, nb, ni);
         tvg_bracket_select_kernel<<<(unsigned)n, 256, 0, st>>>(cand, nb, ni, rows, med, fl);
         tvg_column_select_kernel<<<(unsigned)n, 256, 0, st>>>(ein, rows, n, fl, med);
-        cudaFreeAsync(scr, st);
     }
     tvg_gain_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(med, n, alpha, gain);
     const unsigned gx = (unsigned)((n + 255) / 256);
     const unsigned gy = (unsigned)std::max<long long>(1, std::min<long long>(rows, (16LL * sm_count() + gx - 1) / gx));
     scale_columns_kernel<<<dim3(gx, gy), 256, 0, st>>>((const float2*)d_in, (float2*)d_out, rows, n, gain);
     cudaError_t e = cudaGetLastError();
-    if (own) cudaFreeAsync(own, st);
+    if (scr) cudaFreeAsync(scr, st);
     if (e != cudaSuccess) return cuda_fail(e, "tvg");
     return SAS_OK;
 }
