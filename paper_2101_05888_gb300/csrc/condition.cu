@@ -521,19 +521,26 @@ __global__ void __launch_bounds__(TVG_THREADS, 2) tvg_select_kernel(const float2
 // gives each column a bracket [lo, hi] (bit patterns) that holds the column's
 // middle order statistics with overwhelming probability; one pass over all
 // rows counts the values below lo and collects those inside the bracket
-// (at most TVG_CAP a column); a block per column then selects both middle
+// (at most `cap` <= TVG_CAP a column); a block per column then selects both middle
 // ranks among the collected values.  A column whose bracket misses a middle
 // rank, or whose collection overflowed, is flagged and selected again over
 // all its rows by a block of its own (the three radix levels), so the result
 // is exact in every case.
 constexpr int TVG_CAP = 8192;
-constexpr long long TVG_BRACKET_MIN_ROWS = 8192;    // fewer rows: the three-level select directly (5000 x 2048: as fast)
+// fewer rows: the three-level select directly.  Few columns leave SMs idle, where the
+// bracket's four launches count: 8192 x 1000 takes 120 us with it and 107 without, 10000 x
+// 1000 139 and 136, 16383 x 1000 203 and 255; 8192 x 4096 260 and 351
+constexpr long long TVG_BRACKET_MIN_ROWS = 8192, TVG_BRACKET_MIN_ROWS_NARROW = 12288;
+constexpr int TVG_NARROW = 2048;
 // rows of the sample (about): the bracket holds 4 sqrt(sample) / sample of the rows,
-// which has to stay well below TVG_CAP
+// which has to stay well below the room for candidates: TVG_CAP a column, or 0.3 of the
+// rows below TVG_FEW_ROWS (13 % of them expected, and half as much again six standard
+// deviations up) -- with TVG_CAP there too, a call after a wait, when the allocator has given
+// its memory back, spent 220 of its 738 us on 128 MB for 8192 x 4096 (three levels: 528)
 constexpr long long TVG_SAMPLE = 2048, TVG_SAMPLE_FEW = 1024, TVG_FEW_ROWS = 32768;
 
 __global__ void __launch_bounds__(TVG_THREADS) tvg_collect_kernel(const float2* __restrict__ e, long long rows, int n,
-                                                                  const uint2* __restrict__ bracket,
+                                                                  const uint2* __restrict__ bracket, int cap,
                                                                   unsigned* __restrict__ cand,
                                                                   unsigned* __restrict__ below,
                                                                   unsigned* __restrict__ nin) {
@@ -543,14 +550,14 @@ __global__ void __launch_bounds__(TVG_THREADS) tvg_collect_kernel(const float2* 
     __syncthreads();
     if (col < n) {
         const uint2 br = bracket[col];
-        unsigned* cc = cand + (size_t)col * TVG_CAP;
+        unsigned* cc = cand + (size_t)col * cap;
         unsigned nb = 0u;
         auto put = [&](unsigned bits) {
             if (bits < br.x) {
                 ++nb;
             } else if (bits <= br.y) {
                 const unsigned pos = atomicAdd(&s_cnt[c], 1u);
-                if (pos < (unsigned)TVG_CAP) cc[pos] = bits;
+                if (pos < (unsigned)cap) cc[pos] = bits;
             }
         };
         long long r = threadIdx.x / TVG_COLS;
@@ -592,7 +599,7 @@ __device__ void tvg_block_pick(const unsigned* h, int L, int SH, unsigned* pre, 
 // One column per block: checks the bracket and selects both middle ranks
 // among its collected values (three radix levels on the bit patterns, as
 // above), else flags the column.
-__global__ void __launch_bounds__(256) tvg_bracket_select_kernel(const unsigned* __restrict__ cand,
+__global__ void __launch_bounds__(256) tvg_bracket_select_kernel(const unsigned* __restrict__ cand, int cap,
                                                                  const unsigned* __restrict__ below,
                                                                  const unsigned* __restrict__ nin, long long rows,
                                                                  double* __restrict__ med, int* __restrict__ flags) {
@@ -602,10 +609,10 @@ __global__ void __launch_bounds__(256) tvg_bracket_select_kernel(const unsigned*
     const int col = blockIdx.x;
     const unsigned nb = below[col], ni = nin[col];
     const unsigned R0 = (unsigned)((rows - 1) / 2), R1 = (unsigned)(rows / 2);
-    const bool ok = ni <= (unsigned)TVG_CAP && nb <= R0 && R1 < nb + ni;
+    const bool ok = ni <= (unsigned)cap && nb <= R0 && R1 < nb + ni;
     if (threadIdx.x == 0) flags[col] = ok ? 0 : 1;
     if (!ok) return;
-    for (unsigned t = threadIdx.x; t < ni; t += blockDim.x) v[t] = cand[(size_t)col * TVG_CAP + t];
+    for (unsigned t = threadIdx.x; t < ni; t += blockDim.x) v[t] = cand[(size_t)col * cap + t];
     if (threadIdx.x < 2) {
         pre[threadIdx.x] = 0u;
         rk[threadIdx.x] = (threadIdx.x ? R1 : R0) - nb;
@@ -1080,10 +1087,11 @@ extern "C" int sas_tvg(const void* d_in, void* d_out, int64_t rows, int32_t n, d
     // three-level select runs, which needs none.
     auto up256 = [](size_t x) { return (x + 255) / 256 * 256; };
     const size_t own_bytes = d_median && d_gain ? 0 : up256((sizeof(double) + sizeof(float)) * (size_t)n);
+    const int cap = rows < TVG_FEW_ROWS ? (int)std::min<int64_t>(TVG_CAP, (rows * 3 / 10 + 255) / 256 * 256) : TVG_CAP;
     const size_t o_c = own_bytes + up256(sizeof(uint2) * (size_t)n);
-    const size_t o_b = o_c + sizeof(unsigned) * (size_t)n * TVG_CAP;
+    const size_t o_b = o_c + sizeof(unsigned) * (size_t)n * cap;
     const size_t o_n = o_b + sizeof(unsigned) * n, o_f = o_n + sizeof(unsigned) * n;
-    bool bracketed = rows >= TVG_BRACKET_MIN_ROWS;
+    bool bracketed = rows >= (n < TVG_NARROW ? TVG_BRACKET_MIN_ROWS_NARROW : TVG_BRACKET_MIN_ROWS);
     char* scr = nullptr;
     if (bracketed && cudaMallocAsync((void**)&scr, o_f + sizeof(int) * n, st) != cudaSuccess) {
         (void)cudaGetLastError();
@@ -1114,8 +1122,8 @@ extern "C" int sas_tvg(const void* d_in, void* d_out, int64_t rows, int32_t n, d
         unsigned* ni = reinterpret_cast<unsigned*>(scr + o_n);
         int* fl = reinterpret_cast<int*>(scr + o_f);
         tvg_select_kernel<<<strips, TVG_THREADS, TVG_SMEM, st>>>(ein, m, rstep, n, k_lo, k_hi, nullptr, br);
-        tvg_collect_kernel<<<strips, TVG_THREADS, 0, st>>>(ein, rows, n, br, cand, nb, ni);
-        tvg_bracket_select_kernel<<<(unsigned)n, 256, 0, st>>>(cand, nb, ni, rows, med, fl);
+        tvg_collect_kernel<<<strips, TVG_THREADS, 0, st>>>(ein, rows, n, br, cap, cand, nb, ni);
+        tvg_bracket_select_kernel<<<(unsigned)n, 256, 0, st>>>(cand, cap, nb, ni, rows, med, fl);
         tvg_column_select_kernel<<<(unsigned)n, 256, 0, st>>>(ein, rows, n, fl, med);
     }
     tvg_gain_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(med, n, alpha, gain);

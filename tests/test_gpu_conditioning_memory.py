@@ -59,3 +59,24 @@ def test_gain_without_scratch(rows, n):
     if r.returncode == 77:
         pytest.skip("no pool of a bounded size here")
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("rows,n", [(12287, 9), (12288, 9), (8191, 2048), (8192, 2048), (20000, 5), (32767, 5)])
+def test_select_on_both_sides_of_its_rules(rows, n):
+    """Row counts and widths around the lines of the bracketed select, and columns whose
+    bracket holds more rows than the scratch has room for (half of them equal)."""
+    import paper_2101_05888_gb300 as sas
+    g = torch.Generator(device="cuda")
+    g.manual_seed(rows + n)
+    x = torch.view_as_complex(torch.randn((rows, n, 2), device="cuda", generator=g))
+    x[:, 1] = 0.25 + 0.5j
+    x[::2, 2] = 0.75j                                   # half the rows equal, near the median
+    x[:, 3] = torch.linspace(0.1, 2.0, rows, device="cuda")
+    out, med = torch.empty_like(x), torch.empty(n, dtype=torch.float64, device="cuda")
+    sas.sas_tvg(x, out, rows, n, 0.3, None, med)
+    # re*re + im*im rounded to FP32
+    v = torch.view_as_real(x)
+    p = torch.sort(v[..., 0] * v[..., 0] + v[..., 1] * v[..., 1], dim=0).values.double()
+    ref = 0.5 * (p[(rows - 1) // 2] + p[rows // 2])
+    # PyTorch may fuse the sum (at most one unit in the last place of FP32)
+    assert bool(((med - ref).abs() <= 1.2e-7 * ref).all())
