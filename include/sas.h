@@ -484,11 +484,11 @@ int sas_dpc_model_delays(const sas_dpc_problem* pr, const double* d_vy, const do
  * p_z,i = p_z,0 + sum_{n<i} v_z[n] dt_n.  The normal equations are solved in
  * the equivalent variables (positions p_1 .. p_{P-1} and the last velocity),
  * where they are banded (half-bandwidth 7).  At most max_iter accepted steps;
- * stops when the steps stop shrinking once the loss moves within its rounding
- * (relative 1e-11; a rise within it is accepted from a shrinking step).  h_loss (host,
- * may be NULL): the final Eq. 8 value; h_iters (host, may be NULL): accepted
- * steps.  Synchronises the stream.  Errors: SAS_ERR_ARG, SAS_ERR_OOM,
- * SAS_ERR_CUDA. */
+ * stops when, with the loss moving within its rounding (relative 1e-11; a rise within it
+ * is accepted from a shorter step), a step is below 4e-12 m or three have not been shorter
+ * than the one before them.  h_loss (host, may be NULL): the final Eq. 8 value;
+ * h_iters (host, may be NULL): accepted steps.  Synchronises the stream.  Errors:
+ * SAS_ERR_ARG, SAS_ERR_OOM, SAS_ERR_CUDA. */
 int sas_dpc_solve(const sas_dpc_problem* pr, double* d_vy, double* d_vz, int32_t max_iter, double* h_loss,
                   int32_t* h_iters, void* cuda_stream);
 

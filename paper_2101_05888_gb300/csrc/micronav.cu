@@ -1168,9 +1168,13 @@ extern "C" int sas_dpc_solve(const sas_dpc_problem* pr, double* d_vy, double* d_
     // about 3e-12 of its value, so below LOSS_NOISE it cannot tell two points apart: near
     // the minimum Newton's steps shrink a hundredfold each while the loss moves up or
     // down at random (judged by it, half of them were repeated with growing damping, 20
-    // to 30 trials long).  Such a step is taken when it shrinks, and the search ends
-    // once steps stop shrinking.
-    constexpr double LOSS_NOISE = 1e-11;
+    // to 30 trials long).  Within the noise a step is taken when it is shorter than the one
+    // before, and the search ends with one below STEP_NOISE (at 10 m depth and 100 m paths steps
+    // end at random near 1e-12 m, 100 to 2048 pings alike) or after three that are not
+    // shorter.  (Any shortening counts: with the Huber loss the steps shrink by a third or less
+    // each, and asking for half ended the search up to 1e-8 m, with weak regularisers 5e-5
+    // m, short of the minimum.)
+    constexpr double LOSS_NOISE = 1e-11, STEP_NOISE = 4e-12;
     double mu = 1e-3, last_step = INFINITY;
     int flat = 0;   // trials within the noise that did not shrink
     for (int it = 0; rc == SAS_OK && it < max_iter; ++it) {
@@ -1193,18 +1197,18 @@ extern "C" int sas_dpc_solve(const sas_dpc_problem* pr, double* d_vy, double* d_
             }
             const double step = hacc[2];
             trial = hacc[0];
-            const bool blind = std::fabs(trial - cost) <= LOSS_NOISE * cost, shrinks = step <= 0.5 * last_step;
+            const bool blind = std::fabs(trial - cost) <= LOSS_NOISE * cost, shrinks = step < last_step;
             if (blind && !shrinks) ++flat;
+            done = flat >= 3 || (blind && step <= STEP_NOISE);
             if (trial <= cost || (blind && shrinks)) {
                 std::swap(S.q, q_try);
                 std::swap(cur, nxt);
                 accepted = true;
-                done = step == 0.0 || (blind && std::fabs(cost - trial) <= 1e-14 * cost && !shrinks) || flat >= 3;
+                done = done || step == 0.0 || (blind && !shrinks && std::fabs(cost - trial) <= 1e-14 * cost);
                 last_step = step;
                 mu = std::max(mu / 3.0, 1e-15);
                 break;
             }
-            done = flat >= 3;
             mu *= 4.0;
         }
         if (rc != SAS_OK || !accepted) break;
