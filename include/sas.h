@@ -493,10 +493,10 @@ int sas_dpc_solve(const sas_dpc_problem* pr, double* d_vy, double* d_vz, int32_t
                   int32_t* h_iters, void* cuda_stream);
 
 /* Test hook: the solve inside sas_dpc_solve reduces its unknowns in segments of
- * 64 rows (8 blocks of 8); rows (a power of two in [8, 512]) sets a smaller segment
- * for the following calls of this process (rows / 8 blocks, at least 2, at most 8),
- * so that small problems take several reductions; rows = 0 restores 64.  The
- * result does not depend on it.  Errors: SAS_ERR_ARG. */
+ * eight blocks of 8; rows (a power of two in [8, 512]) sets the segment for the
+ * following calls of this process -- 8 and 16: two blocks, 32: four, 64 and more:
+ * eight -- so that small problems take several reductions; rows = 0 restores
+ * eight.  The result does not depend on it.  Errors: SAS_ERR_ARG. */
 int sas_debug_dpc_solve_chunk(int32_t rows);
 
 #ifdef __cplusplus
