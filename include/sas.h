@@ -342,7 +342,8 @@ int sas_interp_tabulate_mlp(const float* d_theta, int32_t table_n, double prior_
  * kernel computed a Farrow-row index outside the window the host sized for
  * its tile (the kernel clamped it: no access left the buffer, but the
  * result is wrong).
- * After a timeout the results of the calls since the last check are invalid,
+ * After a timeout the results of the calls since the last check are invalid
+ * (an image may hold parts of earlier ones),
  * and a kernel may have left while one of its own bulk copies was still in
  * flight: treat the device state as suspect and recreate the handle (and
  * re-upload the echo) before relying on further results. */

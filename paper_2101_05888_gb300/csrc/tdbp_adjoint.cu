@@ -651,10 +651,6 @@ static int launch_linear_adjoint(sas_geometry_t h, const sas_grid& g, const floa
     core::Setup S;
     int rc = core::prepare(h, g, dim3, 2LL * sm_count(), S, false);
     if (rc != SAS_OK) return rc;
-    if (S.prm.refract && (S.prm.beam || S.prm.vel)) {
-        set_error("the refraction model does not combine with receiver motion or a beam");
-        return SAS_ERR_UNSUPPORTED;
-    }
     SAS_CUDA(cudaMemsetAsync(eadj, 0, sizeof(float2) * (size_t)h->P * h->C * h->Ns, st));
     size_t smem2d = 0;
     if (adjoint2d_plan(h, g, S, smem2d)) {

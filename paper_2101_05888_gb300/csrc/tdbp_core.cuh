@@ -1167,8 +1167,8 @@ __global__ void __launch_bounds__(NTHREADS, 2) tdbp_kernel(const __grid_constant
     float dxv, dyv_c, dv0, dvstep;
     // per slot s: the varying offset d_var(s), |d|^2 and the transmitter
     // differential range of the current ping, held as pairs of slots (2k, 2k+1)
-    // for the packed geometry.  The offsets are formed exactly as the adjoint
-    // kernel forms them, so both evaluate identical paths.
+    // for the packed geometry.  The offsets are formed exactly as adjoint_kernel
+    // forms them, so both evaluate identical paths.
     // (column series: the centre's offset dvc and |d0|^2, and the transmitter's
     // series in half samples)
     float2 dvp[SERIES ? 1 : PX / 2], d2p[SERIES ? 1 : PX / 2], dTp[SERIES ? 1 : PX / 2];
@@ -1771,10 +1771,7 @@ inline void tile_dims(int dim3, int& TXs, int& TYs, int& TZs) {
     }
 }
 
-// Fills the launch description for grid g; slots: CTAs resident on the device,
-// for which the pings of each tile are split (0 = never split); mode: the
-// tdbp_kernel mode the launch runs (sets the Farrow row format).
-// range from which the column series holds on lines of half length ymax, for a
+// Range from which the column series holds on lines of half length ymax, for a
 // point within dmax of the tile centre: the term left out, r |C5| (y / r)^5 with
 // |C5| <= 0.1, stays below 5e-6 rad of carrier phase there (and the line
 // is short against r)
@@ -1788,6 +1785,9 @@ double series_range(sas_geometry_t h, double dmax, double ymax);
 int pick_pings_per_split(long long ntiles, int P, int C, long long slots, bool uneven, double overhead,
                          double sum_cost, long long max_blocks);
 
+// Fills the launch description for grid g; slots: CTAs resident on the device,
+// for which the pings of each tile are split (0 = never split); mode: the
+// tdbp_kernel mode the launch runs (sets the Farrow row format).
 int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long slots, Setup& S, bool need_echo = true,
             int mode = MODE_FORWARD);
 

@@ -216,18 +216,8 @@ static int launch_one(const Setup& S, cudaStream_t st) {
     const bool mv = S.prm.vel != nullptr;
     auto kern = S.prm.beam ? (mv ? tdbp_kernel<ET, DIM3, MODE, true, true> : tdbp_kernel<ET, DIM3, MODE, true, false>)
                            : (mv ? tdbp_kernel<ET, DIM3, MODE, false, true> : tdbp_kernel<ET, DIM3, MODE, false, false>);
-    if constexpr (MODE == MODE_FORWARD) {
-        if (S.prm.refract) {
-            if (S.prm.beam || mv) {
-                set_error("the refraction model does not combine with receiver motion or a beam");
-                return SAS_ERR_UNSUPPORTED;
-            }
-            kern = tdbp_kernel<ET, DIM3, MODE, false, false, true>;
-        }
-    } else if (S.prm.refract) {
-        set_error("the offset gradient is not available with the refraction model");
-        return SAS_ERR_UNSUPPORTED;
-    }
+    if (S.prm.refract)   // without a beam or motion (prepare)
+        kern = tdbp_kernel<ET, DIM3, MODE, false, false, true>;
     if (!S.prm.refract && !S.prm.beam && !mv && S.prm.npos_pad == NPOS_FIXED)
         kern = tdbp_kernel<ET, DIM3, MODE, false, false, false, true>;
     SAS_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S.smem));
