@@ -222,12 +222,6 @@ __device__ __forceinline__ dfl df_sqrt(dfl a) {
     const float e = __fadd_rn(fmaf(-r, r, a.hi), a.lo);   // a - r^2 (exact FMA residual of the high part)
     return df_fast(r, r == 0.0f ? 0.0f : __fmul_rn(e, __fdiv_rn(0.5f, r)));
 }
-// 1 / a: the FP32 reciprocal refined by one Newton step
-__device__ __forceinline__ dfl df_recip(dfl a) {
-    const float q = __fdiv_rn(1.0f, a.hi);
-    const dfl p = df_mul(a, dfl{q, 0.0f}), e = df_add(dfl{1.0f, 0.0f}, dfl{-p.hi, -p.lo});
-    return df_fast(q, __fmul_rn(q, e.hi));
-}
 __device__ __forceinline__ float df_float(dfl x) { return __fadd_rn(x.hi, x.lo); }
 // the double-float nearest a double (host and device)
 __host__ __device__ inline float2 df_split(double v) {

@@ -205,6 +205,13 @@ __device__ __forceinline__ float rcp_sfu(float x) {
     return y;
 }
 
+// x / d: the quotient by the SFU's reciprocal (1e-7) refined by its residual
+__device__ __forceinline__ dfl df_div(dfl x, dfl d) {
+    const float rc = rcp_sfu(d.hi), q = __fmul_rn(x.hi, rc);
+    const dfl p = df_mul(d, dfl{q, 0.0f}), r = df_add(x, dfl{-p.hi, -p.lo});
+    return df_fast(q, __fmul_rn(__fadd_rn(r.hi, r.lo), rc));
+}
+
 // sin and cos on the SFU; callers reduce the argument to [-pi, pi] first
 // (the range on which the SFU approximations are accurate)
 __device__ __forceinline__ void sincos_sfu(float a, float& sn, float& cs) {
@@ -331,10 +338,11 @@ __device__ __forceinline__ PairGeoDF pair_geo_df(const KParams& p, const dfl* X0
 }
 // v != nullptr: the receiver's velocity during reception (Sec. II-D).  With beta = v / c
 // the two-way path s = c tau of the tile centre solves (s - |R_T|)^2 = |R_R - beta s|^2,
-//   s = (|R_T| - rho + sqrt(|W|^2 - (beta^2 |R_R|^2 - rho^2))) / (1 - beta^2),
-// W = R_R - beta |R_T|, rho = R_R . beta (the root's argument without the cancellation
-// of |R_T|^2 against |R_R|^2: s to 5e-12 m at 100 m, for any |beta| < 1 and down to a receiver
-// at the tile centre), and R_R is then taken from the receiver's position at that time (an
+//   s = (|R_T| - rho + sqrt((1 - beta^2) |R_R|^2 + beta^2 |R_T|^2 + rho (rho - 2 |R_T|))) / (1 - beta^2),
+// rho = R_R . beta (the root's argument without |R_T|^2 - |R_R|^2, whose cancellation costs
+// 1e-9 m near the receiver: s to 6e-12 m at 100 m for any |beta| < 1 and down to a receiver at
+// the tile centre; 3e-9 m at 2 m/s, 3e-7 m at 75, where R_R = beta |R_T| and the argument
+// vanishes), and R_R is then taken from the receiver's position at that time (an
 // FP64 fixed point in its place kept the producer warp on the slow FP64 pipe: the stripmap
 // with motion ran at 0.76 of its rate without).
 __device__ __forceinline__ int pair_record_df(const KParams& p, PairGeoDF G, float* rc, int stride,
@@ -351,14 +359,12 @@ __device__ __forceinline__ int pair_record_df(const KParams& p, PairGeoDF G, flo
         auto dot = [](const dfl* x, const dfl* y) {
             return df_add(df_add(df_mul(x[0], y[0]), df_mul(x[1], y[1])), df_mul(x[2], y[2]));
         };
-        const dfl b2 = dot(b, b), rho = dot(G.R, b), n = df_sqrt(dot(G.T, G.T));
-        dfl W[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) W[k] = df_add(G.R[k], df_neg(df_mul(b[k], n)));
-        dfl disc = df_add(dot(W, W), df_add(df_mul(rho, rho), df_neg(df_mul(b2, dot(G.R, G.R)))));
+        const dfl b2 = dot(b, b), rho = dot(G.R, b), T2 = dot(G.T, G.T), n = df_sqrt(T2);
+        const dfl d = df_add(dfl{1.0f, 0.0f}, df_neg(b2));
+        dfl disc = df_add(df_mul(d, dot(G.R, G.R)),
+                          df_add(df_mul(b2, T2), df_mul(rho, df_add(rho, dfl{-2.0f * n.hi, -2.0f * n.lo}))));
         if (disc.hi <= 0.0f) disc = dfl{0.0f, 0.0f};   // zero but for rounding
-        const dfl s = df_mul(df_add(df_add(n, df_neg(rho)), df_sqrt(disc)),
-                             df_recip(df_add(dfl{1.0f, 0.0f}, df_neg(b2))));
+        const dfl s = df_div(df_add(df_add(n, df_neg(rho)), df_sqrt(disc)), d);
 #pragma unroll
         for (int k = 0; k < 3; ++k) G.R[k] = df_add(G.R[k], df_neg(df_mul(b[k], s)));
         rc[F_RV * stride] = df_float(dot(G.R, b));
