@@ -32,6 +32,8 @@ int pick_pings_per_split(long long ntiles, int P, int C, long long slots, bool u
         }
         if (pps == 1) break;
         s = (P - 1) / (pps - 1) + 1;   // the next split with fewer pings a block
+        // within one wave the most splits are the best
+        if (!uneven && s * ntiles < slots) s = (int)std::min<long long>(P, slots / ntiles);
     }
     return best;
 }
