@@ -195,7 +195,7 @@ int prepare(sas_geometry_t h, const sas_grid& g, int dim3, long long slots, Setu
     // tile cost a CTA about 12 pairs' time; adding the parts is another launch, five pairs'
     // time (3 pings x 2 RX -> one tile: 10.0 us in one part, 11.3 us in three).  With a
     // beam the CTAs compute between none and all of their pairs, so whole waves mean
-    // nothing (150 x 4 -> 400 x 300 at 3 cm, 30 degrees: 288 us by whole waves, 257 us now).
+    // nothing (150 x 4 -> 400 x 300 at 3 cm, 30 degrees: 288 us by whole waves, 265 us now).
     const double sum_cost = mode == MODE_FORWARD && need_echo ? 5.0 : 0.0;
     prm.pings_per_split = slots > 0 ? pick_pings_per_split(ntiles, h->P, h->C, slots, prm.beam, 12.0, sum_cost,
                                                            (long long)MAX_WAVES * slots)
